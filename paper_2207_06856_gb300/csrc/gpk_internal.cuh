@@ -113,9 +113,10 @@ int launch_prep_x_f32(Ctx* ctx, const float* X, int64_t N, int64_t N_pad, int d,
 int launch_v_colmax(Ctx* ctx, const float* V, int64_t N, int R, unsigned* cmax_bits, cudaStream_t s);
 int launch_v_pack32(Ctx* ctx, const float* V, int64_t N, int64_t N_pad, int R, const unsigned* cmax_bits,
                     double outputscale, float* V32, float* outscale, cudaStream_t s);
-// Vt rows: [0, R_pad) the (hi) cast, [R_pad, 2 R_pad) the lo parts when vsplit.
+// Vt rows: [0, lo_off) the (hi) cast, [lo_off, 2 lo_off) the lo parts when vsplit
+// (lo_off >= R; zero beyond R in each), zero up to `rows`.
 int launch_v_cast(Ctx* ctx, int prec, int scale_mode, int vsplit, const float* V, int64_t N, int64_t N_pad, int R,
-                  int R_pad, const unsigned* cmax_bits, double outputscale, void* Vt, float* outscale,
+                  int lo_off, int rows, const unsigned* cmax_bits, double outputscale, void* Vt, float* outscale,
                   cudaStream_t s);
 
 // ----------------------------------------------------------------------------
@@ -137,8 +138,8 @@ struct MvmArgs {
 struct TcPlan {
     int n_it = 0, n_jt = 0, n_split = 1, grid = 0, R_pad = 0, k_pad = 0;
     int64_t Nr_pad = 0, Nc_pad = 0;
-    int engine = 0;   // 0: one row tile per item (kmvm_tc.cu); 1: row-tile pairs, transposed P.V (kmvm_tp.cu)
-    int rv = 0;       // engine 1: rows of Vt per tile (R_pad, or 2 R_pad with the hi + lo split)
+    int engine = 0;   // 0: one row tile per item (kmvm_tc.cu); 1: row-tile pairs (kmvm_tp.cu)
+    int rv = 0;       // engine 1: rows of Vt per tile (R, or 2 R with the hi + lo split, padded to 16)
 };
 TcPlan tc_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad);
 int tc_smem_bytes(int k_pad, int R_pad, int vsplit);
@@ -148,9 +149,10 @@ int launch_kmvm_tc(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
                    const CUtensorMap& tmB, const CUtensorMap& tmV, const float* outscale, float* partial,
                    cudaStream_t s);
 
-// Tensor-core engine with the transposed value product (kmvm_tp.cu).  n_it
-// counts pairs of 128-row tiles; the partial buffer is always used.
-bool tp_supported(int k_pad, int R_pad, int vsplit, int psplit);
+// Tensor-core engine over pairs of row tiles (kmvm_tp.cu).  n_it counts pairs
+// of 128-row tiles.
+bool tp_supported(int k_pad, int R_pad, int vsplit);
+int tp_rv(int R, int vsplit);   // rows of Vt per tile
 TcPlan tp_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad, int vsplit);
 size_t tp_partial_floats(const TcPlan& p);
 int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const MvmArgs& a, const CUtensorMap& tmA,

@@ -1,55 +1,57 @@
-// The tensor-core kernel MVM with the transposed value product
-// (Eq. mvm; Sec. 4.1).
+// The tensor-core kernel MVM over pairs of row tiles (Eq. mvm; Sec. 4.1).
 //
 //   out_i = a^2 sum_j k(x_i, x_j) v_j (+ sigma^2 v_i)
 //
-// Same dataflow as kmvm_tc.cu (S = XA_i XB_j^T on the tensor cores with the
-// norm terms folded into the contraction, the kernel function on the special
-// function units, an FP32 accumulation of P V in TMEM), but the value product
-// is computed transposed, for two row tiles at once:
+// S = XA_i XB_j^T on the tensor cores with the norm terms folded into the
+// contraction, the kernel function on the special function units, and an FP32
+// accumulation of P V in TMEM:
 //
-//   O^T (rows r, columns i) += Vt_j (r x 128) . P_j^T      M = 128, N = 256, K = 128
+//   O (rows i, columns r) += P (128 x 128) . Vt_j^T (128 x rv)   M = 128, N = rv, K = 128
 //
-// A tcgen05.mma occupies the issue path for about the same time whatever its
-// N, so the plain orientation (M = 128 rows i, N = R_pad <= 64) spends eight
-// narrow instructions per 128 x 128 tile on P V.  Transposed, one instruction
-// covers 256 rows i, and the right-hand sides' hi and lo parts (rows
-// [0, R_pad) and [R_pad, 2 R_pad) of Vt) share M, so carrying V as hi + lo
-// costs no extra instruction.  P is the B operand and therefore lives in
-// shared memory: each epilogue thread writes its row of P as 16-byte chunks in
-// the 128-byte-swizzled K-major layout the MMA reads (chunk c of row n at
-// physical chunk c ^ (n mod 8)), then fences to the async proxy.  With
-// PSPLIT the kernel tile is carried as hi + lo (Veltkamp split in FP32 on the
-// FMA pipe: hi keeps the operand format's significand, lo = k - hi exactly
-// before its own rounding), and each K-block is multiplied twice.
+// P never leaves TMEM: each epilogue thread reads its columns of a row of S and
+// writes P as packed 16-bit pairs, which is the A operand (.ts form) of the value
+// product.  Shared memory then carries only the operand tiles (X_j for S, Vt_j as
+// the 128-byte-swizzled B operand), whose reads by the tensor core (4 KB + 4 KB per
+// S instruction, 32 rv bytes per value-product instruction) stay far below its 128
+// bytes per cycle.  With P in shared memory (written by the epilogue, read by the
+// tensor core as a 256-row B operand) that port was 87 % busy and bound the kernel.
 //
-// Single-term P is double-buffered per tile (two 64 KB buffers) and its value
-// product issued once the whole tile is stored, so the next tile's S product,
-// issued as soon as the epilogue has read S, never queues behind it.  The
-// hi + lo tile needs twice the bytes: it is staged per 64-column K-block (two
-// 64 KB buffers) and each K-block's product is issued as soon as it is stored.
+// The right-hand sides' hi and lo parts are 2 R of the rv = 16 ceil(2 R / 16)
+// columns of N, so 17 right-hand sides cost N = 48.  With PSPLIT the kernel tile
+// is carried as hi + lo (hi = k rounded to the operand format, lo = k - hi
+// exactly before its own rounding).
 //
 // Work item = (pair of 128-row tiles, column split).  Warps: 0-15 epilogue
-// (warpgroup q handles row tile q & 1, columns [64 (q >> 1), 64 (q >> 1) + 64):
-// four warps per scheduler hide the TMEM and shared-memory latencies behind the
-// special-function work), 16 TMA producer, 17 S issuer and TMEM owner, 18
-// value-product issuer (one issuing warp serialises too many high-latency
-// tcgen05 and mbarrier operations per tile pair; see tp_mma_s).  TMEM: S of
-// tile 0 [0,128), S of tile 1 [128,256), O^T [256,512) (with the FP32 value
-// product, which has no O^T, a second S buffer there).  The epilogue signals
-// each barrier once per warp (after __syncwarp), never once per thread.
-// With HS (GP_MVM_HALF_EXP) the S product accumulates in FP16 and the
-// epilogue evaluates 2^s in FP16 pairs.  Shared memory: the X_j / Vt_j stage ring first, then the two
-// K-block P buffers (32 KB each, 64 KB with the hi + lo split), then the
-// row-tile buffers.  The A operand of the value
-// product spans 128 rows of which the first rv = R_pad (1 + vsplit) hold Vt;
-// the rest reads the following shared memory (the next K-block, stage or P
-// buffer: always inside the allocation) and lands in accumulator rows that
-// are never read.
+// (warpgroup q handles row tile q & 1: four warps per scheduler hide the TMEM
+// latencies behind the special-function work), 16 TMA producer, then the MMA
+// issuers, one or two per row tile.  The two row tiles share nothing but the
+// operand stages, so one's barriers fall into the other's arithmetic.
 //
-// O^T rows are written raw to the partial buffer [n_split][rv][ld_part]; the
-// split reduction sums the column splits and the hi / lo rows, scales by
-// a^2 / s_c and adds sigma^2 v.  Every mbarrier wait is bounded; a wait that
+// What paces the kernel besides the special-function rate is latency: a barrier
+// probe or a tcgen05 operation of a warp beside four busy epilogue warps costs 100-300
+// cycles.  So the epilogue tells the issuers by named barriers (a waiting warp takes
+// no issue slots; as mbarriers polled by the issuers: 0.71 ms instead of 0.62 for the
+// FP16 tile), each with one arrival per warp, and the run-time loops are not
+// unrolled (unrolled, the kernel was 50 KB of code instead of 30 KB: 1.01 ms instead
+// of 0.89 for the hi + lo tile).
+//
+// TMEM, one 512-column allocation per CTA.  WIDE (single-term P, R <= 32): per
+// row tile S (128 columns), P (64) and O (64); S is released as soon as the
+// epilogue has read it, so the next S and the value product run behind the
+// epilogue's arithmetic.  Otherwise hi and lo of P fill exactly the columns of
+// their S and overwrite it in place: a slot is 64 columns of a tile, and each row
+// tile owns a ring of three 64-column buffers (two where O needs 128 columns, R > 32).
+// With the FP32 value product (no P, no O) each row tile has two 128-column buffers.
+//
+// N = 65,536, d = 8, 17 columns, RBF, ms per launch (P in shared memory, one S and
+// one value-product issuer -> this form): FP16 tile 0.774 -> 0.621, hi + lo tile and
+// inputs 1.45 -> 0.88, of which 0.43 is the special-function time of one ex2 a pair.
+// With HS (GP_MVM_HALF_EXP) the S product accumulates in FP16 and the
+// epilogue evaluates 2^s in FP16 pairs.
+//
+// A single column split writes the output directly (scale, noise); several
+// write their hi and lo sums to the partial buffer, which the split reduction
+// adds up in a fixed order.  Every mbarrier wait is bounded; a wait that
 // runs out records DEV_TIMEOUT, drains what was issued, frees TMEM and exits.
 #include "gpk_internal.cuh"
 #include "ptx.cuh"
@@ -64,26 +66,50 @@ constexpr int kBN = 128;
 constexpr int kPairRows = 256;
 constexpr int kMaxStages = 6;
 constexpr int kEpiWarps = 16;
-constexpr int kThreads = (kEpiWarps + 3) * 32;
 constexpr int kTmaWarp = kEpiWarps;
-constexpr int kMmaWarp = kEpiWarps + 1;   // S issuer, TMEM owner
-constexpr int kPvWarp = kEpiWarps + 2;    // value-product issuer
+constexpr int kMmaWarp = kEpiWarps + 1;   // MMA issuers (row tile 0, 1; in place: S of both, then the value products
+                                          // of both); the first owns the TMEM
+constexpr int kMaxBufs = 6;               // S buffers: 2 x ring slot + row tile
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kTmemO = 256;
-constexpr uint32_t kPKBlock = (uint32_t)kPairRows * 128u;   // one 64-column K-block of P: 256 rows x 128 B
 constexpr int kMaxSmemBytes = 227 * 1024;   // opt-in maximum per CTA (512 B kept for static shared memory)
 constexpr uint32_t kSpvVBytes = 128u * 4u * 4u;   // FP32 value product: 128 columns x 4 rows of FP32 v
 
+struct TpSmem {
+    uint32_t xbytes, stage_bytes;
+    int stages, xi_bufs;
+    uint32_t total;   // dynamic shared memory to request (includes 1 KB alignment slack)
+};
+
+__host__ __device__ inline TpSmem tp_smem(int k_pad, int rv) {
+    TpSmem m;
+    m.xbytes = (uint32_t)kBM * (uint32_t)k_pad * 2u;
+    m.stage_bytes = m.xbytes + 2u * (uint32_t)rv * 128u;
+    m.stages = 0;
+    m.xi_bufs = 2;
+    const uint32_t fixed = 1024u + 4u * m.xbytes;
+    for (int s = kMaxStages; s >= 2; --s)
+        if (fixed + (uint32_t)s * m.stage_bytes <= (uint32_t)kMaxSmemBytes - 512u) { m.stages = s; break; }
+    m.total = fixed + (uint32_t)m.stages * m.stage_bytes;
+    return m;
+}
+
 struct TpParams {
     int n_ip, n_jt, n_split, n_items;
-    int k_pad, rv;        // rv: rows of Vt per tile (R_pad, or 2 R_pad with the hi + lo split)
+    int k_pad, rv;        // rv: rows of Vt per tile (N of the value product)
+    int lo_off;           // row of Vt (column of O) where the lo parts start; 0: no lo parts
     int stages, xi_bufs;
-    int psplit;           // 1: P carried as hi + lo
-    int nrhs;             // right-hand sides in use (the FP32 value product: <= 4)
+    TpSmem sm;
+    int nrhs;             // right-hand sides in use
     int spv;              // 1: FP32 value product; the V map is FP32, 128 columns x 4 rows per box
     int diag;             // square Matern-1/2 operator: P_ii = 0 on chip (exact diagonal added later)
     int64_t ld_part;      // n_ip * 256
-    float* partial;       // [n_split][rv][ld_part]
+    float* partial;       // [n_split][hi, lo][nrhs][ld_part]; FP32 value product: [n_split][column half][nrhs][ld_part]
+    // direct output (n_split = 1): out[c][i] = outscale[c] O + noise Vnoise[c][i]
+    float* out;
+    int64_t ld_out, Nr, ld_v;
+    const float* outscale;
+    const float* Vnoise;
+    float noise;
     const uint32_t* mask; // tile skipping: bit jt of word ip * mask_words + jt / 32 set = evaluate, or null
     int mask_words;
     int* err;
@@ -93,35 +119,59 @@ struct TpParams {
 struct TpBarriers {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
-    uint64_t s_full[4];     // [S buffer * 2 + row tile]; a second S buffer only with the FP32 value product
-    uint64_t s_empty[4];
-    uint64_t p_full[2];     // per P buffer: tile slot (single P) or K-block (hi + lo P)
-    uint64_t p_empty[2];
-    uint64_t o_full;
-    uint64_t o_empty;
+    // S and P buffers, [2 x ring slot + row tile]
+    uint64_t s_full[kMaxBufs];
+    uint64_t p_empty[kMaxBufs]; // P consumed by its value product (and, in place, S may be rewritten)
+    uint64_t o_full[2];         // per row tile
     uint64_t xi_full[2];
     uint64_t xi_empty[2];
-    uint64_t drain[2];      // per issuing warp
+    uint64_t drain[4];          // per issuing warp
 };
+
+// Named barriers between the 8 epilogue warps of a row tile (arrive) and its
+// issuer (sync): S read into registers, P stored.  id 0 is __syncthreads.
+constexpr uint32_t kBarThreads = 9 * 32;
+constexpr uint32_t bar_s_read(uint32_t buf) { return 1u + buf; }    // buf = 2 x ring slot + row tile < 4
+constexpr uint32_t bar_p_full(uint32_t buf) { return 5u + buf; }    // < 6
+
+// WIDE (P beside S), in place (P over S, NG buffers per row tile), or FP32 value product.
+enum TpMode { kWide = 0, kInPlace = 1, kSpv = 2 };
+__host__ __device__ constexpr int tp_threads(int mode) { return (kEpiWarps + (mode == kInPlace ? 5 : 3)) * 32; }
+
+// TMEM columns.
+template <int MODE, int NG>
+struct TpTmem {
+    static constexpr uint32_t kS = MODE == kInPlace ? 64u : 128u;          // width of an S buffer
+    static constexpr uint32_t s(uint32_t b, uint32_t w) { return (2u * b + w) * kS; }
+    static constexpr uint32_t p(uint32_t b, uint32_t w) { return MODE == kWide ? 256u + w * 64u : s(b, w); }
+    static constexpr uint32_t o(uint32_t w) { return MODE == kWide ? 384u + w * 64u : 128u * NG + w * (256u - 64u * NG); }
+};
+
+__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// Arrival of an epilogue warp.  A warp whose bounded wait ran out no longer follows
+// the mbarriers, so it waits here instead of running ahead of the barrier's phase.
+__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t threads, bool ok) {
+    if (ok) asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+    else bar_sync(id, threads);
+}
 
 __device__ __forceinline__ void record_error(int* err, int code) { atomicCAS(err, 0, code); }
 
 __device__ __forceinline__ void item_range(const TpParams& p, int item, int& ip, int& sp, int& j0, int& j1) {
-    ip = item % p.n_ip;
-    sp = item / p.n_ip;
-    j0 = (int)(((int64_t)sp * p.n_jt) / p.n_split);
-    j1 = (int)(((int64_t)(sp + 1) * p.n_jt) / p.n_split);
+    // 32-bit: n_split <= 16 and n_jt <= 2^24
+    const uint32_t q = (uint32_t)item / (uint32_t)p.n_ip;
+    sp = (int)q;
+    ip = item - sp * p.n_ip;
+    j0 = (int)(q * (uint32_t)p.n_jt / (uint32_t)p.n_split);
+    j1 = (int)((q + 1u) * (uint32_t)p.n_jt / (uint32_t)p.n_split);
 }
 
 // Whether the column tile jt of row-tile pair ip is evaluated (compact support:
 // a cleared bit means every kernel value of the pair rounds to zero).
 __device__ __forceinline__ bool tile_on(const TpParams& p, int ip, int jt) {
     return !p.mask || ((__ldg(p.mask + (int64_t)ip * p.mask_words + (jt >> 5)) >> (jt & 31)) & 1u);
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
-                 : "memory");
 }
 
 // ---- TMA producer (one thread) ------------------------------------------------
@@ -133,6 +183,7 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
     int ic = 0;
     const uint32_t S = (uint32_t)p.stages;
     const uint32_t kblk = (uint32_t)p.rv * 128u;
+#pragma unroll 1
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
@@ -144,10 +195,11 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
         ptx::tma_load_2d(sX, tmA, &bars.xi_full[xb], 0, ip * kPairRows);
         ptx::tma_load_2d(sX + xbytes, tmA, &bars.xi_full[xb], 0, ip * kPairRows + kBM);
         ++xi_loads;
+#pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
             const uint32_t st = fills % S, u = fills / S;
-            if (u > 0 && !ptx::mbar_wait(&bars.empty[st], (u - 1) & 1, p.limit_ns)) { ok = false; break; }
+            if (u > 0 && !ptx::mbar_wait_sleep(&bars.empty[st], (u - 1) & 1, p.limit_ns)) { ok = false; break; }
             uint8_t* sx = sSt + st * (xbytes + vtbytes);
             ptx::mbar_arrive_expect_tx(&bars.full[st], xbytes + (p.spv ? kSpvVBytes : vtbytes));
             ptx::tma_load_2d(sx, tmB, &bars.full[st], 0, jt * kBN);
@@ -165,132 +217,214 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
         record_error(p.err, DEV_TIMEOUT);
         // Let every copy this thread issued land before the CTA can exit.
         const uint32_t first = fills > S ? fills - S : 0;
+#pragma unroll 1
         for (uint32_t f = first; f < fills; ++f) ptx::mbar_wait(&bars.full[f % S], (f / S) & 1, p.limit_ns);
         const uint32_t nb = (uint32_t)p.xi_bufs;
+#pragma unroll 1
         for (uint32_t q = xi_loads > nb ? xi_loads - nb : 0; q < xi_loads; ++q)
             ptx::mbar_wait(&bars.xi_full[q % nb], (q / nb) & 1, p.limit_ns);
     }
 }
 
-// ---- MMA issuers (two converged warps) ---------------------------------------------
-// Every tcgen05 operation, mbarrier probe and index step of an issuing warp has
-// a latency of the order of a hundred cycles, so one warp issuing both
-// products serialises about thirty of them per tile pair; split in two, the S
-// issuer re-issues S as soon as the epilogue has read it while the other warp
-// is still issuing the previous tile's value product.  Both warps run their
-// loops converged (every decision is warp-uniform) and issue each tcgen05.mma
-// and commit from one elected lane.  The tensor pipe executes what the two
-// warps issue in arrival order; S and O^T live in disjoint TMEM columns.
+// ---- MMA issuers (two converged warps, one per row tile) -----------------------------
+// An issuer waits for the epilogue on named barriers: a waiting warp takes no issue
+// slots, where a warp polling an mbarrier takes them, and queue entries of the unit
+// the special-function instructions go through, from the epilogue warps beside it.
+// The mbarriers it looks at (operand stage landed, P consumed) have normally
+// completed before.  Every decision is warp-uniform; each tcgen05.mma and commit is
+// issued by one elected lane.  The tensor pipe executes what the two warps issue in
+// arrival order; their accumulators are disjoint TMEM columns.
+//
+// A bounded wait that runs out makes the role go on without further waits or tensor
+// work: it still meets its named barriers, so that every warp reaches the end.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
     return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, limit_ns));
 }
 
-// S issuer: for each column tile, S = XA_i XB_j^T for both row tiles once both
-// S buffers have been read (s_empty) and the stage has landed (full).
-__device__ void tp_mma_s(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
-                         uint32_t xbytes, uint32_t vtbytes, uint32_t tmem, uint32_t id_s) {
-    const uint32_t arow = (uint32_t)p.k_pad * 2u;                            // 32, 64 or 128 bytes
-    const uint32_t swz = (arow == 32) ? 6u : (arow == 64 ? 4u : 2u);
-    const int ksteps = p.k_pad / 16;
-    const uint32_t S = (uint32_t)p.stages;
-    const uint32_t aSt = ptx::smem_u32(sSt);
-    const uint32_t stage_bytes = xbytes + vtbytes;
-    const uint32_t hi_x = ptx::smem_desc_hi(8u * arow, swz);
-    uint32_t g = 0, st = 0, ph = 0;   // tiles issued; stage ring slot and its fill parity
-    int ic = 0;
+// Walks the column tiles whose S is issued; runs one tile ahead of the value
+// product, across items.
+template <int MODE, int NG>
+struct TpSIssue {
+    using T = TpTmem<MODE, NG>;
+    const TpParams& p;
+    TpBarriers& bars;
+    uint32_t aSt, aXi0, xbytes, stage_bytes, arow, hi_x, tmem, id, w;
+    int item, jt, j1, ip, xb;
+    uint32_t ic = 0;            // items entered
+    uint32_t st = 0, ph = 0;    // stage ring slot and its fill parity
+    uint32_t b = 0, bph = 1;    // buffer ring slot; parity of its last release (first round: passes at once)
+    bool have = true;           // a tile is selected (its stage has landed)
     bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x, ++ic) {
-        int ip, sp, j0, j1;
-        item_range(p, item, ip, sp, j0, j1);
-        const int xb = p.xi_bufs == 2 ? (ic & 1) : 0;
-        const int use = p.xi_bufs == 2 ? (ic >> 1) : ic;
-        if (!warp_wait(&bars.xi_full[xb], use & 1, p.limit_ns)) { ok = false; break; }
-        ptx::tc_fence_after();
-        const uint32_t aXi = ptx::smem_u32(sXi) + (uint32_t)xb * 2u * xbytes;
-        for (int jt = j0; jt < j1; ++jt) {
-            if (!tile_on(p, ip, jt)) continue;
-            // S buffer of this tile (two with the FP32 value product, whose O^T columns are free)
-            const uint32_t nb = p.spv ? 2u : 1u, buf = g % nb, use = g / nb;
-            if (use > 0 && !(warp_wait(&bars.s_empty[2 * buf], (use - 1) & 1, p.limit_ns) &&
-                             warp_wait(&bars.s_empty[2 * buf + 1], (use - 1) & 1, p.limit_ns))) { ok = false; break; }
-            if (!warp_wait(&bars.full[st], ph, p.limit_ns)) { ok = false; break; }
-            ptx::tc_fence_after();
-            const uint32_t aXj = aSt + st * stage_bytes;
-            for (int w = 0; w < 2; ++w) {
-                for (int kk = 0; kk < ksteps; ++kk) {
-                    const uint32_t koff = (uint32_t)kk * 32u;
-                    ptx::mma_f16_ss_elect(tmem + buf * 256u + (uint32_t)w * 128u,
-                                          ptx::smem_desc_at(hi_x, aXi + (uint32_t)w * xbytes + koff),
-                                          ptx::smem_desc_at(hi_x, aXj + koff), id_s, kk > 0 ? 1u : 0u);
-                }
-                ptx::mma_commit_elect(&bars.s_full[2 * buf + w]);
-            }
-            if (++st == S) { st = 0; ph ^= 1u; }
-            ++g;
-        }
-        if (!ok) break;
-        ptx::mma_commit_elect(&bars.xi_empty[xb]);   // the row tiles' last use in this item
+
+    __device__ TpSIssue(const TpParams& p_, TpBarriers& bars_, const uint8_t* sSt, const uint8_t* sXi, uint32_t xbytes_,
+                        uint32_t stage_bytes_, uint32_t tmem_, uint32_t id_, uint32_t w_)
+        : p(p_), bars(bars_), xbytes(xbytes_), stage_bytes(stage_bytes_), tmem(tmem_), id(id_), w(w_) {
+        aSt = ptx::smem_u32(sSt);
+        aXi0 = ptx::smem_u32(sXi) + w * xbytes;
+        arow = (uint32_t)p.k_pad * 2u;   // 32, 64 or 128 bytes
+        hi_x = ptx::smem_desc_hi(8u * arow, (arow == 32) ? 6u : (arow == 64 ? 4u : 2u));
+        item = (int)blockIdx.x - (int)gridDim.x;
+        jt = j1 = 0;
     }
-    ptx::mma_commit_elect(&bars.drain[0]);
-    warp_wait(&bars.drain[0], 0, p.limit_ns);
-    if (!ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
+    // Select the next evaluated tile; have = false after the last.
+    __device__ __forceinline__ void next() {
+        ++jt;
+#pragma unroll 1
+        while (have) {
+            if (jt < j1) {
+                if (tile_on(p, ip, jt)) {
+                    ok = ok && warp_wait(&bars.full[st], ph, p.limit_ns);
+                    return;
+                }
+                ++jt;
+                continue;
+            }
+            if (ic > 0 && ok) ptx::mma_commit_elect(&bars.xi_empty[xb]);   // the row tile's last use in its item
+            item += (int)gridDim.x;
+            if (item >= p.n_items) { have = false; return; }
+            int sp;
+            item_range(p, item, ip, sp, jt, j1);
+            xb = p.xi_bufs == 2 ? (int)(ic & 1u) : 0;
+            ok = ok && warp_wait(&bars.xi_full[xb], (p.xi_bufs == 2 ? ic >> 1 : ic) & 1u, p.limit_ns);
+            ++ic;
+        }
+    }
+    // S of columns [h kS, (h + 1) kS) of the selected tile into the ring's next buffer.
+    __device__ __forceinline__ void issue(uint32_t h) {
+        if (ok) {
+            const uint32_t aXi = aXi0 + (uint32_t)xb * 2u * xbytes, aXj = aSt + st * stage_bytes + h * T::kS * arow;
+            ptx::tc_fence_after();
+#pragma unroll 1
+            for (uint32_t k = 0; k < arow; k += 32u)   // K-steps of 16 elements
+                ptx::mma_f16_ss_elect(tmem + T::s(b, w), ptx::smem_desc_at(hi_x, aXi + k),
+                                      ptx::smem_desc_at(hi_x, aXj + k), id, k > 0 ? 1u : 0u);
+            ptx::mma_commit_elect(&bars.s_full[2u * b + w]);
+        }
+        if (++b == NG) { b = 0; bph ^= 1u; }
+    }
+    __device__ __forceinline__ void next_stage() {
+        if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
+    }
+};
+
+// The value product of one slot: O (+)= P Vt^T over 128 (WIDE) or 64 columns.
+template <int MODE, int NG, int PSPLIT>
+__device__ __forceinline__ void tp_value_product(uint32_t tO, uint32_t tP, uint32_t aV, uint32_t kblk, uint32_t id_pv,
+                                                 uint32_t acc) {
+    const uint32_t hi_128 = ptx::smem_desc_hi(1024u, 2u);
+    const uint64_t dV = ptx::smem_desc_at(hi_128, aV);
+    ptx::tc_fence_after();
+    if constexpr (MODE == kWide) {
+        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP, dV, id_pv, acc);
+        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP + 32u, ptx::smem_desc_at(hi_128, aV + kblk), id_pv, 1u);
+    } else {
+        ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP, dV, id_pv, acc);
+        if constexpr (PSPLIT) ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP + 16u, dV, id_pv, 1u);
+    }
 }
 
-// Value-product issuer: O^T += Vt_j P_j^T for each tile (single P: the whole
-// tile once both K-blocks are stored; hi + lo P: per K-block), then releases
-// the P buffer and the stage; O^T is handed to the epilogue after an item.
-template <int PSPLIT>
-__device__ void tp_mma_pv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sP,
-                          uint32_t xbytes, uint32_t vtbytes, uint32_t tmem, uint32_t id_pv) {
-    const uint32_t S = (uint32_t)p.stages;
-    const uint32_t aSt = ptx::smem_u32(sSt);
-    const uint32_t aP = ptx::smem_u32(sP);
-    const uint32_t stage_bytes = xbytes + vtbytes;
-    const uint32_t kblk = (uint32_t)p.rv * 128u;
-    const uint32_t hi_128 = ptx::smem_desc_hi(1024u, 2u);
-    uint32_t g = 0, st = 0, ph = 0;
-    int ic = 0;
-    bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x, ++ic) {
+// WIDE, issuer of row tile w: S(t + 1) once the epilogue holds S(t) in registers,
+// then O += P(t) Vt^T once it has stored P(t).  In place, value-product issuer
+// (the S issuer of tp_issuer_s refills the buffers): O += P(q) Vt^T for each slot.
+template <int MODE, int NG, int PSPLIT>
+__device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi, uint32_t xbytes,
+                          uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t id_pv, uint32_t w) {
+    using T = TpTmem<MODE, NG>;
+    TpSIssue<MODE, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+    const uint32_t aV0 = ptx::smem_u32(sSt) + xbytes, kblk = (uint32_t)p.rv * 128u;
+    const uint32_t tO = tmem + T::o(w);
+    uint32_t st = 0, ph = 0, b = 0;
+    if constexpr (MODE == kWide) {
+        si.next();
+        if (si.have) { si.issue(0); si.next_stage(); }
+    }
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
-        if (ic > 0 && !warp_wait(&bars.o_empty, (ic - 1) & 1, p.limit_ns)) { ok = false; break; }
-        uint32_t t = 0;   // evaluated tiles of this item
-        for (int jt = j0; jt < j1 && ok; ++jt) {
+        uint32_t acc = 0;   // 0 for the item's first product (the epilogue has read O of the last item before
+                            // it stores this item's first P)
+#pragma unroll 1
+        for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
-            // Vt_j of this stage: landed before S of this tile was issued (already complete)
-            if (!warp_wait(&bars.full[st], ph, p.limit_ns)) { ok = false; break; }
-            for (uint32_t kb = 0; kb < (PSPLIT ? 2u : 1u); ++kb) {
-                const uint32_t buf = PSPLIT ? kb : (g & 1u);
-                const uint32_t par = PSPLIT ? (g & 1u) : ((g >> 1) & 1u);
-                if (!warp_wait(&bars.p_full[buf], par, p.limit_ns)) { ok = false; break; }
-                ptx::tc_fence_after();
-                const uint32_t aV = aSt + st * stage_bytes + xbytes + kb * kblk;
-                const uint32_t aPb = aP + buf * 2u * kPKBlock;
-                // single P: K-blocks 0, 1 of the tile (8 steps); hi + lo: hi then lo of K-block kb
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const uint32_t kk = (uint32_t)(q & 3) * 32u, hq = (uint32_t)(q >> 2);
-                    const uint32_t aVq = PSPLIT ? aV + kk : aV + hq * kblk + kk;
-                    const uint32_t aPq = aPb + hq * kPKBlock + kk;
-                    ptx::mma_f16_ss_elect(tmem + kTmemO, ptx::smem_desc_at(hi_128, aVq),
-                                          ptx::smem_desc_at(hi_128, aPq), id_pv,
-                                          (t > 0 || kb > 0 || q > 0) ? 1u : 0u);
+            const uint32_t aV = aV0 + st * stage_bytes;
+            if constexpr (MODE == kWide) {
+                // (this tile's stage landed before its S was issued)
+                bar_sync(bar_s_read(w), kBarThreads);
+                si.next();
+                if (si.have) { si.issue(0); si.next_stage(); }
+                bar_sync(bar_p_full(w), kBarThreads);
+                if (si.ok) {
+                    tp_value_product<MODE, NG, PSPLIT>(tO, tmem + T::p(0, w), aV, kblk, id_pv, acc);
+                    ptx::mma_commit_elect(&bars.p_empty[w]);
                 }
-                ptx::mma_commit_elect(&bars.p_empty[buf]);      // this P buffer may be rewritten
+            } else {
+                si.ok = si.ok && warp_wait(&bars.full[st], ph, p.limit_ns);
+#pragma unroll
+                for (uint32_t h = 0; h < 2; ++h) {
+                    bar_sync(bar_p_full(2u * b + w), kBarThreads);
+                    if (si.ok) {
+                        tp_value_product<MODE, NG, PSPLIT>(tO, tmem + T::p(b, w), aV + h * kblk, kblk, id_pv,
+                                                           h > 0 ? 1u : acc);
+                        ptx::mma_commit_elect(&bars.p_empty[2u * b + w]);
+                    }
+                    if (++b == NG) b = 0;
+                }
             }
-            if (!ok) break;
-            ptx::mma_commit_elect(&bars.empty[st]);             // X_j and Vt_j of this stage are consumed
-            if (++st == S) { st = 0; ph ^= 1u; }
-            ++t;
-            ++g;
+            if (si.ok) ptx::mma_commit_elect(&bars.empty[st]);   // this row tile is done with X_j and Vt_j of the stage
+            if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
+            acc = 1;
         }
-        if (!ok) break;
-        ptx::mma_commit_elect(&bars.o_full);
+        if (si.ok) ptx::mma_commit_elect(&bars.o_full[w]);
     }
-    ptx::mma_commit_elect(&bars.drain[1]);
-    warp_wait(&bars.drain[1], 0, p.limit_ns);
-    if (!ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
+    const uint32_t dr = MODE == kInPlace ? 2u + w : w;
+    ptx::mma_commit_elect(&bars.drain[dr]);
+    warp_wait(&bars.drain[dr], 0, p.limit_ns);
+    if (!si.ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
+}
+
+// In place, S issuer of row tile w: S of each slot (64 columns of a tile) once the
+// value product of the slot NG before it in the ring has completed.
+template <int NG>
+__device__ void tp_issuer_s(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
+                            uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
+    TpSIssue<kInPlace, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+#pragma unroll 1
+    for (si.next(); si.have && si.ok; si.next()) {
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            si.ok = si.ok && warp_wait(&bars.p_empty[2u * si.b + w], si.bph, p.limit_ns);
+            si.issue(h);
+        }
+        si.next_stage();
+    }
+    ptx::mma_commit_elect(&bars.drain[w]);
+    warp_wait(&bars.drain[w], 0, p.limit_ns);
+    if (!si.ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
+}
+
+// Issuer of row tile w for the FP32 value product: S only, two buffers.
+template <int NG>
+__device__ void tp_issuer_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
+                              uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
+    TpSIssue<kSpv, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+    uint32_t n = 0;
+    for (si.next(); si.have; si.next(), ++n) {
+        if (n >= NG) bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
+        si.issue(0);
+        si.next_stage();
+    }
+    for (uint32_t q = 0; q < (n < NG ? n : NG); ++q) {   // the epilogue's last reads
+        if (n >= NG) {
+            bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
+            if (++si.b == NG) si.b = 0;
+        } else {
+            bar_sync(bar_s_read(2u * q + w), kBarThreads);
+        }
+    }
+    ptx::mma_commit_elect(&bars.drain[w]);
+    warp_wait(&bars.drain[w], 0, p.limit_ns);
+    if (!si.ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
 }
 
 template <int BF16>
@@ -304,162 +438,179 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     }
 }
 
-// 32 columns [32 h, 32 h + 32) of this thread's P row: kernel values, packed
-// in pairs (and, with PSPLIT, split hi + lo first), stored as four 16-byte
-// chunks of the swizzled K-major layout of K-block buffer pkb.
+// (l0, l1) = (k0, k1) minus the two halves of u, exact: one mixed-precision FMA each
+// (1.004 -> 0.930 ms for the hi + lo MVM at N = 65,536, 17 columns, against unpacking
+// to FP32 and subtracting).
+template <int BF16>
+__device__ __forceinline__ void sub_packed(float k0, float k1, uint32_t u, float& l0, float& l1) {
+    if constexpr (BF16) {
+        l0 = k0 - __uint_as_float(u << 16);
+        l1 = k1 - __uint_as_float(u & 0xffff0000u);
+    } else {
+        asm("{\n\t.reg .b16 a, b, m;\n\t"
+            "mov.b32 {a, b}, %2;\n\t"
+            "mov.b16 m, 0xBC00;\n\t"   // -1
+            "fma.rn.f32.f16 %0, a, m, %3;\n\t"
+            "fma.rn.f32.f16 %1, b, m, %4;\n\t}"
+            : "=f"(l0), "=f"(l1)
+            : "r"(u), "f"(k0), "f"(k1));
+    }
+}
+
+// Kernel values of 32 columns [col0, col0 + 32) of this thread's row, packed in
+// pairs (and, with PSPLIT, split: pl holds the lo parts).
 template <int KIND, int BF16, int PSPLIT>
-__device__ __forceinline__ void tp_chunk(const uint32_t (&r)[32], int h, int row, bool dtile, uint32_t pkb,
-                                         uint32_t nsw) {
-    // Veltkamp factor 2^(24 - t) + 1 leaves t significant bits in hi: 11 (FP16) or 8 (BF16)
-    constexpr float kSplit = BF16 ? 65537.0f : 8193.0f;
-    uint32_t pk[16];
-    uint32_t pl[PSPLIT ? 16 : 1];
+__device__ __forceinline__ void tp_values(const uint32_t (&r)[32], int col0, int row, bool dtile, uint32_t (&pk)[16],
+                                          uint32_t (&pl)[16]) {
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
         float k0 = kernel_from_s<KIND>(__uint_as_float(r[2 * e]));
         float k1 = kernel_from_s<KIND>(__uint_as_float(r[2 * e + 1]));
         if constexpr (KIND == GP_KERNEL_MATERN12) {
             if (dtile) {
-                const int col = h * 32 + 2 * e;
+                const int col = col0 + 2 * e;
                 if (col == row) k0 = 0.0f;
                 if (col + 1 == row) k1 = 0.0f;
             }
         }
+        pk[e] = pack2<BF16>(k0, k1);
         if constexpr (PSPLIT) {
-            // explicit round-to-nearest operations: no contraction into FMAs
-            const float c0 = __fmul_rn(k0, kSplit), c1 = __fmul_rn(k1, kSplit);
-            const float h0 = __fsub_rn(c0, __fsub_rn(c0, k0)), h1 = __fsub_rn(c1, __fsub_rn(c1, k1));
-            pk[e] = pack2<BF16>(h0, h1);
-            pl[e] = pack2<BF16>(__fsub_rn(k0, h0), __fsub_rn(k1, h1));
-        } else {
-            pk[e] = pack2<BF16>(k0, k1);
+            float l0, l1;
+            sub_packed<BF16>(k0, k1, pk[e], l0, l1);
+            pl[e] = pack2<BF16>(l0, l1);
         }
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const uint32_t c = (uint32_t)((h & 1) * 4 + q);
-        const uint32_t off = (c ^ nsw) << 4;
-        st_shared_v4(pkb + off, pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-        if constexpr (PSPLIT) st_shared_v4(pkb + kPKBlock + off, pl[4 * q], pl[4 * q + 1], pl[4 * q + 2], pl[4 * q + 3]);
-    }
 }
 
-// Half-precision kernel evaluation (RBF, FP16): the S tile comes from the
-// MMA as FP16 (one rounding of the exp2 argument), is loaded packed in pairs,
-// and 2^s is evaluated for both halves of a register by one ex2.approx.f16x2,
-// whose output is already the packed FP16 P the value product reads: no
-// FP32 -> FP16 conversion, one SFU instruction per two kernel values.
-// 32 columns [32 h, 32 h + 32) of this thread's P row from 16 packed S
-// registers, stored as four 16-byte chunks.
-__device__ __forceinline__ void tp_chunk_h(const uint32_t* r, int h, uint32_t pkb, uint32_t nsw) {
-    uint32_t pk[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) pk[e] = ptx::ex2_h2(r[e]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const uint32_t c = (uint32_t)((h & 1) * 4 + q);
-        st_shared_v4(pkb + ((c ^ nsw) << 4), pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-    }
-}
-
-template <int KIND, int BF16, int PSPLIT, int HS>
-__device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, const uint8_t* sP, uint32_t tmem, int wg, int wq,
-                            int lane) {
-    const int tl = wg & 1, ch = wg >> 1;              // row tile of the pair, column half (= K-block)
+template <int KIND, int BF16, int PSPLIT, int HS, int MODE, int NG>
+__device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, int wg, int wq, int lane) {
+    using T = TpTmem<MODE, NG>;
+    constexpr int H = kBN / (int)T::kS;
+    const int tl = wg & 1, ch = wg >> 1;              // row tile of the pair, half of a slot's columns
     const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
     const int row = wq * 32 + lane;                   // row within the tile
-    const uint32_t nrow = (uint32_t)(tl * kBM + row); // row of the P operand (0..255)
-    const uint32_t nsw = nrow & 7u;
-    // P buffers are 64 KB: single P: [tile slot][K-block]; hi + lo: [K-block][hi, lo]
-    const uint32_t aProw = ptx::smem_u32(sP) + nrow * 128u;
-    uint32_t gt = 0;
+    uint32_t b = 0, ph = 0;                           // buffer ring slot and its fill parity
     int ic = 0;
     bool ok = true;
+#pragma unroll 1
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
         const int it = 2 * ip + tl;   // this warpgroup's row tile
-        uint32_t t = 0;               // evaluated tiles of this item
+        bool any = false;             // a tile of this item was evaluated
+#pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
-            const uint32_t g = gt + t;
-            if (!__all_sync(0xffffffffu, ptx::mbar_wait(&bars.s_full[tl], g & 1, p.limit_ns))) { ok = false; break; }
-            ptx::tc_fence_after();
-            const uint32_t tS = tmem + lane_off + (uint32_t)tl * 128u + (uint32_t)ch * 64u;
             const bool dtile = (KIND == GP_KERNEL_MATERN12) && p.diag && (jt == it);
-            uint32_t ra[32], rb[HS ? 1 : 32];
-            if constexpr (HS) {
-                ptx::tmem_ld32_pack16(tS, ra);     // 64 FP16 columns in 32 registers
-                ptx::tmem_wait_ld();
-                ptx::tmem_reg_fence(ra);
-            } else {
-                ptx::tmem_ld32(tS, ra);
-                ptx::tmem_ld32(tS + 32u, rb);
-                ptx::tmem_wait_ld();
-                ptx::tmem_reg_fence(ra);
-                ptx::tmem_reg_fence(rb);
-            }
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars.s_empty[tl]);   // this warp's part of S is in registers
-            uint32_t buf;
-            if constexpr (PSPLIT) {
-                // K-block buffer ch is free once the previous tile's product of it is done
-                buf = (uint32_t)ch;
-                if (g >= 1 && !__all_sync(0xffffffffu, ptx::mbar_wait(&bars.p_empty[buf], (g - 1) & 1, p.limit_ns))) {
-                    ok = false;
-                    break;
-                }
-            } else {
-                // tile slot g & 1 is free once the product of tile g - 2 is done
-                buf = g & 1u;
-                if (g >= 2 &&
-                    !__all_sync(0xffffffffu, ptx::mbar_wait(&bars.p_empty[buf], ((g >> 1) - 1) & 1, p.limit_ns))) {
-                    ok = false;
-                    break;
-                }
-            }
-            const uint32_t pkb = aProw + buf * 2u * kPKBlock + (PSPLIT ? 0u : (uint32_t)ch * kPKBlock);
-            if constexpr (HS) {
-                tp_chunk_h(ra, 2 * ch, pkb, nsw);
-                tp_chunk_h(ra + 16, 2 * ch + 1, pkb, nsw);
-            } else {
-                tp_chunk<KIND, BF16, PSPLIT>(ra, 2 * ch, row, dtile, pkb, nsw);
-                tp_chunk<KIND, BF16, PSPLIT>(rb, 2 * ch + 1, row, dtile, pkb, nsw);
-            }
-            ptx::fence_proxy_async_smem();        // P stores -> visible to the tensor core
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars.p_full[buf]);
-            ++t;
-        }
-        if (!ok) break;
-        // O^T read-out: lanes [0, rv) are the rows of Vt; this warpgroup's 64 columns.
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&bars.o_full, ic & 1, p.limit_ns))) { ok = false; break; }
-        ptx::tc_fence_after();
-        if (wq * 32 < p.rv) {   // warp-uniform
-            const int r = wq * 32 + lane;
-            float* dst = p.partial + ((int64_t)sp * p.rv + r) * p.ld_part + (int64_t)ip * kPairRows + tl * kBM + ch * 64;
-            for (int h = 0; h < 2; ++h) {
-                uint32_t o[32];
-                if (t > 0) {
-                    ptx::tmem_ld32(tmem + lane_off + kTmemO + (uint32_t)(tl * kBM + ch * 64 + h * 32), o);
-                    ptx::tmem_wait_ld();
-                    ptx::tmem_reg_fence(o);
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const uint32_t buf = 2u * b + (uint32_t)tl;
+                ok = ok && warp_wait(&bars.s_full[buf], ph, p.limit_ns);
+                ptx::tc_fence_after();
+                const uint32_t tS = tmem + lane_off + T::s(b, (uint32_t)tl) + (uint32_t)ch * (T::kS / 2u);
+                uint32_t pk[16], pl[16];
+                if constexpr (MODE == kWide) {
+                    const uint32_t tP = tmem + lane_off + T::p(b, (uint32_t)tl) + (uint32_t)ch * 32u;
+                    uint32_t ra[32], rb[HS ? 1 : 32];
+                    if constexpr (HS) {
+                        // Half-precision kernel evaluation (RBF, FP16): the S tile comes from the
+                        // MMA as FP16 (one rounding of the exp2 argument), is loaded packed in pairs,
+                        // and 2^s is evaluated for both halves of a register by one ex2.approx.f16x2,
+                        // whose output is already the packed FP16 P the value product reads: no
+                        // FP32 -> FP16 conversion, one SFU instruction per two kernel values.
+                        ptx::tmem_ld32_pack16(tS, ra);     // 64 FP16 columns in 32 registers
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_reg_fence(ra);
+                    } else {
+                        ptx::tmem_ld32(tS, ra);
+                        ptx::tmem_ld32(tS + 32u, rb);
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_reg_fence(ra);
+                        ptx::tmem_reg_fence(rb);
+                    }
+                    ptx::tc_fence_before();
+                    bar_arrive(bar_s_read((uint32_t)tl), kBarThreads, ok);   // S is in registers
+                    if constexpr (HS) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) pk[e] = ptx::ex2_h2(ra[e]);
+                    } else {
+                        tp_values<KIND, BF16, 0>(ra, ch * 64, row, dtile, pk, pl);
+                    }
+                    // P is free once the value product of the previous tile is done (first use: at once)
+                    ok = ok && warp_wait(&bars.p_empty[buf], ph ^ 1u, p.limit_ns);
+                    ptx::tc_fence_after();
+                    ptx::tmem_st16(tP, pk);
+                    if constexpr (HS) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) pk[e] = ptx::ex2_h2(ra[16 + e]);
+                    } else {
+                        tp_values<KIND, BF16, 0>(rb, ch * 64 + 32, row, dtile, pk, pl);
+                    }
+                    ptx::tmem_st16(tP + 16u, pk);
                 } else {
+                    // in place: hi over the first 16 of this thread's 32 columns of S, lo over the others
+                    uint32_t ra[32];
+                    if constexpr (HS) {
+                        ptx::tmem_ld16_pack16(tS, pk);     // 32 FP16 columns in 16 registers
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_reg_fence(pk);
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) o[q] = 0u;   // every tile of the item was skipped
+                        for (int e = 0; e < 16; ++e) pk[e] = ptx::ex2_h2(pk[e]);
+                    } else {
+                        ptx::tmem_ld32(tS, ra);
+                        ptx::tmem_wait_ld();
+                        ptx::tmem_reg_fence(ra);
+                        tp_values<KIND, BF16, PSPLIT>(ra, h * 64 + ch * 32, row, dtile, pk, pl);
+                    }
+                    ptx::tmem_st16(tS, pk);
+                    if constexpr (PSPLIT) ptx::tmem_st16(tS + 16u, pl);
                 }
-                float4* d4 = reinterpret_cast<float4*>(dst + h * 32);
+                ptx::tmem_wait_st();
+                ptx::tc_fence_before();
+                bar_arrive(bar_p_full(buf), kBarThreads, ok);
+                if (++b == NG) { b = 0; ph ^= 1u; }
+            }
+            any = true;
+        }
+        // O read-out: lanes are rows of the tile; this warpgroup's half of the right-hand sides.
+        ok = ok && warp_wait(&bars.o_full[tl], ic & 1, p.limit_ns);
+        ptx::tc_fence_after();
+        const int half = (p.nrhs + 1) >> 1;
+        const int c0 = ch * half, c1 = ch ? p.nrhs : half;
+        const uint32_t tO = tmem + lane_off + T::o((uint32_t)tl);
+        const int64_t i = (int64_t)ip * kPairRows + tl * kBM + row;
+#pragma unroll 1
+        for (int c = c0; c < c1; c += 8) {   // warp-uniform
+            uint32_t oh[8], ol[8];
+            if (any) {
+                ptx::tmem_ld8(tO + (uint32_t)c, oh);
+                ptx::tmem_ld8(tO + (uint32_t)(p.lo_off + c), ol);
+                ptx::tmem_wait_ld();
+                ptx::tmem_reg_fence(oh);
+                ptx::tmem_reg_fence(ol);
+            } else {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    d4[q] = make_float4(__uint_as_float(o[4 * q]), __uint_as_float(o[4 * q + 1]),
-                                        __uint_as_float(o[4 * q + 2]), __uint_as_float(o[4 * q + 3]));
+                for (int e = 0; e < 8; ++e) oh[e] = ol[e] = 0u;   // every tile of the item was skipped
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int cc = c + e;
+                if (cc < c1) {
+                    const float hi = __uint_as_float(oh[e]), lo = __uint_as_float(ol[e]);
+                    if (p.n_split > 1) {   // rows [split][hi, lo][column], summed in this order
+                        const int parts = p.lo_off ? 2 : 1;
+                        float* o = p.partial + ((int64_t)sp * parts * p.nrhs + cc) * p.ld_part + i;
+                        *o = hi;
+                        if (p.lo_off) o[(int64_t)p.nrhs * p.ld_part] = lo;
+                    } else if (i < p.Nr) {
+                        float v = (p.lo_off ? hi + lo : hi) * __ldg(p.outscale + cc);
+                        if (p.noise != 0.0f) v = fmaf(p.noise, __ldg(p.Vnoise + (int64_t)cc * p.ld_v + i), v);
+                        p.out[(int64_t)cc * p.ld_out + i] = v;
+                    }
+                }
             }
         }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&bars.o_empty);
-        gt += t;
+        ptx::tc_fence_before();   // ordered before this item's successor by the next P's barrier
     }
     if (!ok) record_error(p.err, DEV_TIMEOUT);
 }
@@ -467,11 +618,11 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, const uint8_t* 
 // The FP32 value product (GP_MVM_FP32_PV, 1 to 4 right-hand sides): the
 // epilogue keeps its kernel values in FP32 and forms sum_j k_ij v_j itself
 // with FP32 FMAs, v_j read in FP32 from the stage (TMA box of 128 columns x 4
-// rows; this warpgroup's 64 columns; broadcast 16-byte reads).  No P in shared
-// memory and no value-product MMAs: a tensor-core product with 1 to 4 useful
+// rows; this warpgroup's 64 columns; broadcast 16-byte reads).  No P and no
+// value-product MMAs: a tensor-core product with 1 to 4 useful
 // rows of its M = 128 would cost as much as one with 64.  Each warp releases
 // the stage after its reads (16 arrivals), and writes its row sums of the item
-// to the partial rows ch * R_pad + r, which the split reduction adds up.
+// to the partial rows ch * R + r, which the split reduction adds up.
 template <int KIND, int RN>
 __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, uint32_t xbytes,
                                 uint32_t vtbytes, uint32_t tmem, int wg, int wq, int lane) {
@@ -480,10 +631,9 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
     const int row = wq * 32 + lane;
     const uint32_t S = (uint32_t)p.stages;
     const uint32_t stage_bytes = xbytes + vtbytes;
-    const int Rp = p.rv >> 1;
-    constexpr int R = RN;   // columns 1, 2 or 4 (3 runs as 4: the fourth row of v is zero)
     uint32_t gt = 0, st = 0, ph = 0;
     bool ok = true;
+#pragma unroll 1
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
@@ -492,17 +642,14 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
 #pragma unroll
         for (int r = 0; r < RN; ++r) acc[r] = 0.0f;
         uint32_t t = 0;
+#pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
             const uint32_t g = gt + t, buf = g & 1u;
             // hinted waits: a spinning warp would take the issue slots of the warps computing
             // beside it and of the S issuer on its scheduler (this epilogue is issue-bound)
-            if (!__all_sync(0xffffffffu,
-                            ptx::mbar_wait_sleep(&bars.s_full[2 * buf + tl], (g >> 1) & 1, p.limit_ns) &&
-                                ptx::mbar_wait_sleep(&bars.full[st], ph, p.limit_ns))) {
-                ok = false;
-                break;
-            }
+            ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait_sleep(&bars.s_full[2 * buf + tl], (g >> 1) & 1, p.limit_ns) &&
+                                                   ptx::mbar_wait_sleep(&bars.full[st], ph, p.limit_ns));
             ptx::tc_fence_after();
             const uint32_t tS = tmem + lane_off + buf * 256u + (uint32_t)tl * 128u + (uint32_t)ch * 64u;
             const bool dtile = (KIND == GP_KERNEL_MATERN12) && p.diag && (jt == it);
@@ -518,8 +665,7 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
                 ptx::tmem_reg_fence(rr);
                 if (hh == 1) {
                     ptx::tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(&bars.s_empty[2 * buf + tl]);
+                    bar_arrive(bar_s_read(2u * buf + (uint32_t)tl), kBarThreads, ok);
                 }
 #pragma unroll
                 for (int c4 = 0; c4 < 4; ++c4) {      // 16-byte chunk c: columns [8 c, 8 c + 8) of the 64
@@ -556,44 +702,19 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
             if (++st == S) { st = 0; ph ^= 1u; }
             ++t;
         }
-        if (!ok) break;
 #pragma unroll
-        for (int r = 0; r < RN; ++r)
-            p.partial[((int64_t)sp * p.rv + ch * Rp + r) * p.ld_part + (int64_t)ip * kPairRows + tl * kBM + row] =
-                acc[r];
+        for (int r = 0; r < RN; ++r)   // RN = 1, 2 or 4 (3 runs as 4: the fourth row of v is zero)
+            if (r < p.nrhs)
+                p.partial[((int64_t)(2 * sp + ch) * p.nrhs + r) * p.ld_part + (int64_t)ip * kPairRows + tl * kBM + row] =
+                    acc[r];
         gt += t;
     }
     if (!ok) record_error(p.err, DEV_TIMEOUT);
 }
 
-struct TpSmem {
-    uint32_t xbytes, vtbytes, stage_bytes, pbuf;
-    int stages, xi_bufs;
-    uint32_t total;   // dynamic shared memory to request (includes 1 KB alignment slack)
-};
-
-__host__ __device__ inline TpSmem tp_smem(int k_pad, int rv, int psplit) {
-    TpSmem m;
-    m.xbytes = (uint32_t)kBM * (uint32_t)k_pad * 2u;
-    m.vtbytes = 2u * (uint32_t)rv * 128u;
-    m.stage_bytes = m.xbytes + m.vtbytes;
-    m.pbuf = (uint32_t)(1 + psplit) * kPKBlock;
-    const uint32_t fixed = 1024u + 4u * kPKBlock;   // two 64 KB P buffers
-    m.stages = 0;
-    m.xi_bufs = 2;
-    for (int xb = 2; xb >= 1 && m.stages < 3; --xb) {
-        const uint32_t xi = (uint32_t)xb * 2u * m.xbytes;
-        int st = 0;
-        for (int s = kMaxStages; s >= 2; --s)
-            if (fixed + xi + (uint32_t)s * m.stage_bytes <= (uint32_t)kMaxSmemBytes - 512u) { st = s; break; }
-        if (st > m.stages) { m.stages = st; m.xi_bufs = xb; }
-    }
-    m.total = fixed + (uint32_t)m.xi_bufs * 2u * m.xbytes + (uint32_t)m.stages * m.stage_bytes;
-    return m;
-}
-
-template <int KIND, int BF16, int PSPLIT, int HS, int SPV>
-__global__ void __launch_bounds__(kThreads, 1)
+// MODE and NG as in TpTmem (in place: NG = 3 when O takes 64 columns per row tile, 2 when it takes 128).
+template <int KIND, int BF16, int PSPLIT, int HS, int SPV, int MODE, int NG>
+__global__ void __launch_bounds__(tp_threads(MODE), 1)
 kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmV, const TpParams p) {
     extern __shared__ uint8_t dsm[];
@@ -601,31 +722,30 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __shared__ uint32_t tmem_slot;
 
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~uintptr_t(1023));
-    const TpSmem m = tp_smem(p.k_pad, p.rv, PSPLIT);
+    const TpSmem& m = p.sm;
     uint8_t* sSt = base;
-    uint8_t* sP = base + (uint32_t)p.stages * m.stage_bytes;
-    uint8_t* sXi = sP + 4u * kPKBlock;
+    uint8_t* sXi = base + (uint32_t)p.stages * m.stage_bytes;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxStages; ++s) {
-            ptx::mbar_init(&bars.full[s], 1);
-            ptx::mbar_init(&bars.empty[s], SPV ? kEpiWarps : 1);   // FP32 product: each epilogue warp
+#pragma unroll 1
+        for (int b = 0; b < kMaxStages; ++b) {
+            ptx::mbar_init(&bars.full[b], 1);
+            ptx::mbar_init(&bars.empty[b], SPV ? kEpiWarps : 2);   // the two value products; FP32: each epilogue warp
         }
-        for (int b = 0; b < 4; ++b) {
+#pragma unroll 1
+        for (int b = 0; b < kMaxBufs; ++b) {
             ptx::mbar_init(&bars.s_full[b], 1);
-            ptx::mbar_init(&bars.s_empty[b], 8);                // the 8 warps of a row tile (one arrival each)
-        }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(&bars.xi_full[b], 1);
-            ptx::mbar_init(&bars.xi_empty[b], 1);
-            ptx::mbar_init(&bars.p_full[b], PSPLIT ? 8 : 16);   // K-block: 2 warpgroups; tile: all 4 (per warp)
             ptx::mbar_init(&bars.p_empty[b], 1);
         }
-        ptx::mbar_init(&bars.o_full, 1);
-        ptx::mbar_init(&bars.o_empty, kEpiWarps);
-        ptx::mbar_init(&bars.drain[0], 1);
-        ptx::mbar_init(&bars.drain[1], 1);
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+            ptx::mbar_init(&bars.xi_full[b], 1);
+            ptx::mbar_init(&bars.xi_empty[b], 2);
+            ptx::mbar_init(&bars.o_full[b], 1);
+            ptx::mbar_init(&bars.drain[b], 1);
+            ptx::mbar_init(&bars.drain[2 + b], 1);
+        }
         ptx::fence_mbar_init();
     }
     if (warp == kTmaWarp && lane == 0) {
@@ -640,19 +760,29 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tmem = tmem_slot;
 
     if (warp == kTmaWarp) {
-        if (lane == 0) tp_producer(p, &tmA, &tmB, &tmV, bars, sSt, sXi, m.xbytes, m.vtbytes);
+        if (lane == 0) tp_producer(p, &tmA, &tmB, &tmV, bars, sSt, sXi, m.xbytes, m.stage_bytes - m.xbytes);
         __syncwarp();
-    } else if (warp == kMmaWarp) {
-        tp_mma_s(p, bars, sSt, sXi, m.xbytes, m.vtbytes, tmem,
-                 HS ? ptx::idesc_f16_dh(kBM, kBN) : ptx::idesc_f16(kBM, kBN, BF16));
-    } else if (warp == kPvWarp) {
-        if constexpr (!SPV)
-            tp_mma_pv<PSPLIT>(p, bars, sSt, sP, m.xbytes, m.vtbytes, tmem, ptx::idesc_f16(kBM, kPairRows, BF16));
+    } else if (warp >= kMmaWarp) {
+        constexpr int kW = (int)TpTmem<MODE, NG>::kS;
+        const uint32_t id_s = HS ? ptx::idesc_f16_dh(kBM, kW) : ptx::idesc_f16(kBM, kW, BF16);
+        const uint32_t w = (uint32_t)(warp - kMmaWarp) & 1u;
+        if constexpr (MODE == kInPlace) {
+            if (warp < kMmaWarp + 2)
+                tp_issuer_s<NG>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
+            else
+                tp_issuer<MODE, NG, PSPLIT>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
+                                            ptx::idesc_f16(kBM, p.rv, BF16), w);
+        } else if constexpr (SPV > 0)
+            tp_issuer_spv<NG>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
+        else
+            tp_issuer<MODE, NG, PSPLIT>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
+                                        ptx::idesc_f16(kBM, p.rv, BF16), w);
     } else {
         if constexpr (SPV > 0)
-            tp_epilogue_spv<KIND, SPV>(p, bars, sSt, m.xbytes, m.vtbytes, tmem, warp >> 2, warp & 3, lane);
+            tp_epilogue_spv<KIND, SPV>(p, bars, sSt, m.xbytes, m.stage_bytes - m.xbytes, tmem, warp >> 2, warp & 3,
+                                       lane);
         else
-            tp_epilogue<KIND, BF16, PSPLIT, HS>(p, bars, sP, tmem, warp >> 2, warp & 3, lane);
+            tp_epilogue<KIND, BF16, PSPLIT, HS, MODE, NG>(p, bars, tmem, warp >> 2, warp & 3, lane);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -660,30 +790,46 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (warp == kMmaWarp) ptx::tmem_dealloc(tmem, kTmemCols);
 }
 
+template <int KIND, int BF16, int PSPLIT, int HS, int SPV, int MODE, int NG>
+cudaError_t launch_tp_mode(const TcPlan& plan, const TpParams& prm, const CUtensorMap& a, const CUtensorMap& b,
+                           const CUtensorMap& v, cudaStream_t s) {
+    const TpSmem& m = prm.sm;
+    auto kfn = kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV, MODE, NG>;
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.total);
+    if (e != cudaSuccess) return e;
+    kfn<<<plan.grid, tp_threads(MODE), m.total, s>>>(a, b, v, prm);
+    return cudaGetLastError();
+}
+
 template <int KIND, int BF16, int PSPLIT, int HS = 0, int SPV = 0>
 cudaError_t launch_tp_typed(const TcPlan& plan, const TpParams& prm, const CUtensorMap& a, const CUtensorMap& b,
                             const CUtensorMap& v, cudaStream_t s) {
-    const TpSmem m = tp_smem(prm.k_pad, prm.rv, PSPLIT);
-    auto kfn = kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.total);
-    if (e != cudaSuccess) return e;
-    kfn<<<plan.grid, kThreads, m.total, s>>>(a, b, v, prm);
-    return cudaGetLastError();
+    if constexpr (SPV > 0) {
+        return launch_tp_mode<KIND, BF16, PSPLIT, HS, SPV, kSpv, 2>(plan, prm, a, b, v, s);
+    } else {
+        if (prm.rv > 64) return launch_tp_mode<KIND, BF16, PSPLIT, HS, 0, kInPlace, 2>(plan, prm, a, b, v, s);
+        if constexpr (PSPLIT) return launch_tp_mode<KIND, BF16, PSPLIT, HS, 0, kInPlace, 3>(plan, prm, a, b, v, s);
+        else return launch_tp_mode<KIND, BF16, PSPLIT, HS, 0, kWide, 1>(plan, prm, a, b, v, s);
+    }
 }
 
 }  // namespace
 
-bool tp_supported(int k_pad, int R_pad, int vsplit, int psplit) {
-    const int rv = R_pad * (1 + vsplit);
-    return k_pad <= 64 && rv <= 128 && rv % 32 == 0 && tp_smem(k_pad, rv, psplit).stages >= 2;
+// The operand sets this engine takes (rp: right-hand sides padded to 16, hi and
+// lo padded separately); the others run on the one-tile engine.
+bool tp_supported(int k_pad, int R_pad, int vsplit) {
+    const int rp = R_pad * (1 + vsplit);
+    return k_pad <= 64 && rp <= (k_pad == 64 ? 64 : 128) && rp % 32 == 0;
 }
+
+int tp_rv(int R, int vsplit) { return ((R * (1 + vsplit) + 15) / 16) * 16; }
 
 TcPlan tp_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad, int vsplit) {
     TcPlan p;
     p.engine = 1;
     p.k_pad = k_pad;
     p.R_pad = ((R + 15) / 16) * 16;
-    p.rv = p.R_pad * (1 + vsplit);
+    p.rv = tp_rv(R, vsplit);
     const int n_it = (int)((Nr + kBM - 1) / kBM);
     p.n_it = (n_it + 1) / 2;                  // pairs of row tiles
     p.n_jt = (int)((Nc + kBN - 1) / kBN);
@@ -701,7 +847,7 @@ TcPlan tp_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad, int vsp
         const int64_t waves = (items + G - 1) / G;
         const int64_t tiles = (p.n_jt + sp - 1) / sp;
         double cost = (double)waves * (double)(tiles + 2);
-        cost += 0.05 * (double)sp * (double)p.n_it * 2.0 * (double)p.rv / (double)G / 64.0;
+        cost += 0.05 * (double)sp * (double)p.n_it * 2.0 * (double)(p.R_pad * (1 + vsplit)) / (double)G / 64.0;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = sp; }
     }
     p.n_split = best;
@@ -722,16 +868,25 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
     prm.n_items = plan.n_it * plan.n_split;
     prm.k_pad = plan.k_pad;
     prm.rv = plan.rv;
-    prm.psplit = L.psplit;
+    prm.lo_off = L.vsplit ? a.R : 0;
     prm.nrhs = a.R;
     prm.spv = L.fp32_pv ? 1 : 0;
-    const TpSmem m = tp_smem(plan.k_pad, plan.rv, L.psplit);
+    if (!tp_supported(plan.k_pad, plan.R_pad, L.vsplit)) return GP_ERR_UNSUPPORTED;
+    const TpSmem m = tp_smem(plan.k_pad, plan.rv);
+    if (m.stages < 2) return GP_ERR_UNSUPPORTED;
     prm.stages = m.stages;
     prm.xi_bufs = m.xi_bufs;
-    if (!tp_supported(plan.k_pad, plan.R_pad, plan.rv / plan.R_pad - 1, L.psplit)) return GP_ERR_UNSUPPORTED;
+    prm.sm = m;
     prm.diag = a.diag_coef != 0.0f ? 1 : 0;
     prm.ld_part = plan.Nr_pad;
     prm.partial = partial;
+    prm.out = a.out;
+    prm.ld_out = a.ld_out;
+    prm.Nr = a.Nr;
+    prm.ld_v = a.Nc;
+    prm.outscale = outscale;
+    prm.Vnoise = a.Vnoise;
+    prm.noise = a.noise + a.diag_coef;
     prm.mask = mask;
     prm.mask_words = (plan.n_jt + 31) / 32;
     prm.err = ctx->dev_err;
@@ -751,7 +906,7 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
                          : launch_tp_typed<K, 0, 0>(plan, prm, tmA, tmB, tmV, s);                    \
         break;
     const bool spv = L.fp32_pv != 0;
-    if (spv && (bf || L.psplit || hs || a.R > 4 || plan.rv != 2 * plan.R_pad)) return GP_ERR_UNSUPPORTED;
+    if (spv && (bf || L.psplit || hs || a.R > 4 || !L.vsplit)) return GP_ERR_UNSUPPORTED;
     if (hs) {
         e = launch_tp_typed<GP_KERNEL_RBF, 0, 0, 1>(plan, prm, tmA, tmB, tmV, s);
     } else if (spv) {
@@ -781,10 +936,10 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
     prof_end(ctx, s);
     ctx->launches++;
     if (e != cudaSuccess) return GP_ERR_CUDA;
-    // splits x {hi, lo} rows: partial[s][part * R_pad + c] = partial'[s * parts + part][c]
-    const int parts = plan.rv / plan.R_pad;
-    return launch_split_reduce(ctx, partial, plan.n_split * parts, plan.Nr_pad, a.Nr, a.R, plan.R_pad, outscale,
-                               0.0f, a.noise + a.diag_coef, a.Vnoise, a.Nc, a.out, a.ld_out, s);
+    if (!spv && plan.n_split == 1) return GP_OK;
+    // splits times hi and lo rows (times the two column halves of the FP32 value product)
+    return launch_split_reduce(ctx, partial, plan.n_split * (L.vsplit ? 2 : 1), plan.Nr_pad, a.Nr, a.R, a.R, outscale, 0.0f,
+                               a.noise + a.diag_coef, a.Vnoise, a.Nc, a.out, a.ld_out, s);
 }
 
 }  // namespace gpk

@@ -139,13 +139,12 @@ static int kop_plan(const Ctx* ctx, KOp& op, const gp_hyp_t* hyp, int64_t Nr, in
         const int Rc = R < 64 ? R : 64;
         const int Rp = ((Rc + 15) / 16) * 16;
         const OperandLayout probe = make_layout(hyp->d, op.prec, xsplit, 1, psplit);
-        // Pair engine (transposed value product) unless asked otherwise or the
-        // operands do not fit its shared-memory plan.  There FP16 carries v as
-        // hi + lo (the lo rows share the MMA's M dimension) and, with
-        // GP_MVM_PSPLIT, the kernel tile as hi + lo too.
+        // Pair engine unless asked otherwise or the operands do not fit its
+        // plan.  There FP16 carries v as hi + lo (both in the columns of one
+        // value product) and, with GP_MVM_PSPLIT, the kernel tile as hi + lo too.
         const int want_psplit = bf ? psplit : ((flags & GP_MVM_PSPLIT) ? 1 : 0);
         const bool pair = !(flags & GP_MVM_ONE_TILE) && probe.k_pad != 0 &&
-                          tp_supported(probe.k_pad, Rp, bf ? vsplit : 1, want_psplit);
+                          tp_supported(probe.k_pad, Rp, bf ? vsplit : 1);
         if (pair && !bf) {
             vsplit = 1;
             psplit = want_psplit;
@@ -275,7 +274,8 @@ int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_o
         } else {
             TcPlan pl = op.tp;
             pl.R_pad = ((rc + 15) / 16) * 16;
-            if (pl.engine == 1) pl.rv = pl.R_pad * (op.lay.vsplit ? 2 : 1);
+            if (pl.engine == 1) pl.rv = tp_rv(rc, op.lay.vsplit);
+            const int vrows = pl.engine == 1 ? pl.rv : (op.lay.vsplit ? 2 : 1) * pl.R_pad;
             GPK_TRY(launch_v_colmax(ctx, Vc, op.Nc, rc, op.cmax, s));
             if (pl.engine == 1 && op.lay.fp32_pv) {
                 // FP32 value product: v in FP32 (4 rows, in the FP16 Vt buffer's space, which
@@ -289,18 +289,18 @@ int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_o
                 continue;
             }
             GPK_TRY(launch_v_cast(ctx, op.prec, (op.flags & GP_MVM_SCALE_SQRT_N) ? 1 : 0, op.lay.vsplit, Vc, op.Nc,
-                                  pl.Nc_pad, rc, pl.R_pad, op.cmax, op.a2, op.Vt, op.outscale, s));
+                                  pl.Nc_pad, rc, pl.engine == 1 && op.lay.vsplit ? rc : pl.R_pad, vrows, op.cmax, op.a2, op.Vt,
+                                  op.outscale, s));
             const CUtensorMapDataType dt =
                 op.prec == GP_PREC_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-            const uint64_t vrows = (uint64_t)(op.lay.vsplit ? 2 : 1) * pl.R_pad;
             if (pl.engine == 1) {
                 // one box carries the hi and lo rows of a 64-column K-block
-                GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, vrows, pl.Nc_pad * 2, 64, (uint32_t)pl.rv,
+                GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, (uint64_t)vrows, pl.Nc_pad * 2, 64, (uint32_t)pl.rv,
                                        CU_TENSOR_MAP_SWIZZLE_128B));
                 GPK_TRY(launch_kmvm_tp(ctx, pl, op.lay, a, op.tmA, op.tmB, op.tmV, op.outscale, op.partial,
                                        op.skip ? op.mask : nullptr, s));
             } else {
-                GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, vrows, pl.Nc_pad * 2, 64, pl.R_pad,
+                GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, (uint64_t)vrows, pl.Nc_pad * 2, 64, pl.R_pad,
                                        CU_TENSOR_MAP_SWIZZLE_128B));
                 GPK_TRY(launch_kmvm_tc(ctx, pl, op.lay, a, op.tmA, op.tmB, op.tmV, op.outscale, op.partial, s));
             }

@@ -216,10 +216,11 @@ int launch_v_colmax(Ctx* ctx, const float* V, int64_t N, int R, unsigned* cmax_b
     return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
 }
 
-// Cast V (N x R col-major FP32) to Vt (R_pad x N_pad, operand type), each
+// Cast V (N x R col-major FP32) to Vt (rows x N_pad, operand type), each
 // column scaled by s_c; outscale[c] = a^2 / s_c.  Two elements per thread.
+// blockIdx.y < lo_off: vector c's hi row (and its lo row); beyond: a zero row.
 template <typename T>
-__global__ void v_cast_kernel(const float* __restrict__ V, int64_t N, int64_t N_pad, int R, int R_pad,
+__global__ void v_cast_kernel(const float* __restrict__ V, int64_t N, int64_t N_pad, int R, int lo_off,
                               const unsigned* __restrict__ cmax_bits, int scale_mode, int vsplit, float a2,
                               T* __restrict__ Vt, float* __restrict__ outscale, int* err) {
     const int c = blockIdx.y;
@@ -242,8 +243,16 @@ __global__ void v_cast_kernel(const float* __restrict__ V, int64_t N, int64_t N_
             }
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) outscale[c] = (c < R) ? os : 0.0f;
     const int64_t j = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (c >= lo_off) {
+        const int row = c + (vsplit ? lo_off : 0);
+        if (j < N_pad) {
+            Vt[(int64_t)row * N_pad + j] = to_op<T>(0.0f);
+            Vt[(int64_t)row * N_pad + j + 1] = to_op<T>(0.0f);
+        }
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) outscale[c] = (c < R) ? os : 0.0f;
     if (j >= N_pad) return;
     const float* v = V + (int64_t)c * N;
     const float v0 = (c < R && j < N) ? v[j] * sc : 0.0f;
@@ -253,7 +262,7 @@ __global__ void v_cast_kernel(const float* __restrict__ V, int64_t N, int64_t N_
     o[0] = h0;
     o[1] = h1;
     if (vsplit) {
-        T* q = Vt + (int64_t)(R_pad + c) * N_pad + j;
+        T* q = Vt + (int64_t)(lo_off + c) * N_pad + j;
         q[0] = to_op<T>(v0 - from_op<T>(h0));
         q[1] = to_op<T>(v1 - from_op<T>(h1));
     }
@@ -289,17 +298,17 @@ int launch_v_pack32(Ctx* ctx, const float* V, int64_t N, int64_t N_pad, int R, c
 }
 
 int launch_v_cast(Ctx* ctx, int prec, int scale_mode, int vsplit, const float* V, int64_t N, int64_t N_pad, int R,
-                  int R_pad, const unsigned* cmax_bits, double outputscale, void* Vt, float* outscale,
+                  int lo_off, int rows, const unsigned* cmax_bits, double outputscale, void* Vt, float* outscale,
                   cudaStream_t s) {
     const int threads = 256;
     const int64_t blocks = (N_pad / 2 + threads - 1) / threads;
-    dim3 grid((unsigned)blocks, (unsigned)R_pad);
+    dim3 grid((unsigned)blocks, (unsigned)(vsplit ? rows - lo_off : rows));
     if (prec == GP_PREC_BF16) {
-        v_cast_kernel<__nv_bfloat16><<<grid, threads, 0, s>>>(V, N, N_pad, R, R_pad, cmax_bits, scale_mode, vsplit,
+        v_cast_kernel<__nv_bfloat16><<<grid, threads, 0, s>>>(V, N, N_pad, R, lo_off, cmax_bits, scale_mode, vsplit,
                                                               (float)outputscale, (__nv_bfloat16*)Vt,
                                                               outscale, ctx->dev_err);
     } else {
-        v_cast_kernel<__half><<<grid, threads, 0, s>>>(V, N, N_pad, R, R_pad, cmax_bits, scale_mode, vsplit,
+        v_cast_kernel<__half><<<grid, threads, 0, s>>>(V, N, N_pad, R, lo_off, cmax_bits, scale_mode, vsplit,
                                                        (float)outputscale, (__half*)Vt, outscale,
                                                        ctx->dev_err);
     }

@@ -265,12 +265,6 @@ __device__ __forceinline__ void wprime(float s, float h, float& w, float& hk) {
     }
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
 template <int KIND>
 __device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, uint32_t tmem, int q, int wq, int lane,
                              double* red) {
@@ -331,7 +325,7 @@ __device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, uint32_t tme
             for (int c = 0; c < 16; ++c) dst[(int64_t)c * p.N_pad] = __uint_as_float(o[c]);
         } else {
             uint32_t o[8];
-            tmem_ld8(tmem + lane_off + kColO + (uint32_t)c0, o);
+            ptx::tmem_ld8(tmem + lane_off + kColO + (uint32_t)c0, o);
             ptx::tmem_wait_ld();
             ptx::tmem_reg_fence(o);
 #pragma unroll
@@ -688,7 +682,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     ctx->launches += 3;
     if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
     GPK_TRY(launch_v_colmax(ctx, Vb, N, d + 1, cmv, s));
-    GPK_TRY(launch_v_cast(ctx, GP_PREC_FP16, 0, 1, Vb, N, pl.Nc_pad, d + 1, pl.rx, cmv, 1.0, Xt, xs, s));
+    GPK_TRY(launch_v_cast(ctx, GP_PREC_FP16, 0, 1, Vb, N, pl.Nc_pad, d + 1, pl.rx, 2 * pl.rx, cmv, 1.0, Xt, xs, s));
 
     CUtensorMap tmUW, tmWU, tmXt;
     const uint32_t hrow = (uint32_t)pl.kh * 2u;

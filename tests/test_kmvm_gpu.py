@@ -498,3 +498,23 @@ def test_fp32_value_product_refusals(ctx):
         _run(ctx, X, V[:2], kern, ls, a2, s2, "bf16", flags=gpk.MVM_FP32_PV)
     with pytest.raises(gpk.GPKError):       # not with the hi + lo kernel tile
         _run(ctx, X, V[:2], kern, ls, a2, s2, "fp16", flags=gpk.MVM_FP32_PV | gpk.MVM_PSPLIT)
+
+
+@pytest.mark.parametrize("R", [1, 8, 9, 16, 24, 31, 32, 33, 47, 49, 64])
+@pytest.mark.parametrize("N", [127, 129, 257, 641])
+@pytest.mark.parametrize("mode", ["fp16", "hilo", "bf16", "half_exp"])
+def test_pair_engine_tile_edges(ctx, mode, N, R):
+    """Edges of the pair engine's plan: row tiles and pairs that end one short of
+    or one past a tile, one and several column splits, the value product's width
+    (hi and lo of R columns padded to 16) at its steps, O of one (R <= 32) and of
+    two TMEM column blocks (R > 32), with P beside S and over S.  Tolerances as
+    above; with kernel tile, inputs and vectors as hi + lo each source keeps 22
+    significant bits or more and at most 641 terms are summed in FP32 (1e-4)."""
+    from paper_2207_06856_gb300 import gpk
+    X, V, _, ls, a2, s2 = workloads.random_problem(N, 8, R, seed=N + 5 * R, kernel=0)
+    prec, fl, tol = {"fp16": ("fp16", 0, TOL["fp16"]),
+                     "hilo": ("fp16", gpk.MVM_PSPLIT | gpk.MVM_XSPLIT, 1e-4),
+                     "bf16": ("bf16", 0, TOL["bf16"]),
+                     "half_exp": ("fp16", gpk.MVM_HALF_EXP, TOL["fp16"])}[mode]
+    got = _run(ctx, X, V, 0, ls, a2, s2, prec, flags=fl)
+    assert _colerr(got, _ref(X, V, 0, ls, a2, s2)) <= tol
