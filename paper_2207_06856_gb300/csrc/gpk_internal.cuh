@@ -161,7 +161,7 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
 
 // SIMT FP32 engine (kmvm_simt.cu).  Scaled FP32 inputs with row stride dp.
 struct SimtPlan {
-    int dp = 0, R_pad = 0, n_rowblk = 0, n_split = 1;
+    int dp = 0, R = 0, R_pad = 0, n_rowblk = 0, n_split = 1;
 };
 SimtPlan simt_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int d, int R);
 size_t simt_partial_floats(const SimtPlan& p, int64_t Nr);

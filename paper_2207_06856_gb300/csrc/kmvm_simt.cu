@@ -115,7 +115,7 @@ kmvm_simt_kernel(const float* __restrict__ Xr, const float* __restrict__ Xc, con
                     out[(int64_t)c * ld_out + i1] = v;
                 }
             } else {
-                float* pp = partial + ((int64_t)blockIdx.y * RPM + c) * ld_part;
+                float* pp = partial + ((int64_t)blockIdx.y * R + c) * ld_part;
                 if (i0 < Nr) pp[i0] = s0;
                 if (i1 < Nr) pp[i1] = s1;
             }
@@ -134,6 +134,31 @@ __global__ void split_reduce_kernel(const float* __restrict__ partial, int n_spl
     if (i >= Nr || c >= R) return;
     float s = 0.0f;
     for (int sp = 0; sp < n_split; ++sp) s += partial[((int64_t)sp * RP + c) * ld_part + i];
+    float v = s * (outscale ? outscale[c] : scale_const);
+    if (noise != 0.0f) v = fmaf(noise, Vnoise[(int64_t)c * ld_v + i], v);
+    out[(int64_t)c * ld_out + i] = v;
+}
+
+// The same for many splits of few rows, where one thread per output would walk
+// them all: 32 rows x 8 groups per block, group g sums splits g, g + 8, .. and the
+// groups are added in order.
+__global__ void __launch_bounds__(256)
+split_reduce_wide_kernel(const float* __restrict__ partial, int n_split, int64_t ld_part, int RP, int64_t Nr, int R,
+                         const float* __restrict__ outscale, float scale_const, float noise,
+                         const float* __restrict__ Vnoise, int64_t ld_v, float* __restrict__ out, int64_t ld_out) {
+    __shared__ float sg[8][32];
+    const int c = blockIdx.y, l = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + l;
+    float s = 0.0f;
+    if (i < Nr) {
+#pragma unroll 8
+        for (int sp = g; sp < n_split; sp += 8) s += partial[((int64_t)sp * RP + c) * ld_part + i];
+    }
+    sg[g][l] = s;
+    __syncthreads();
+    if (g != 0 || i >= Nr) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sg[q][l];
     float v = s * (outscale ? outscale[c] : scale_const);
     if (noise != 0.0f) v = fmaf(noise, Vnoise[(int64_t)c * ld_v + i], v);
     out[(int64_t)c * ld_out + i] = v;
@@ -177,6 +202,7 @@ cudaError_t simt_dispatch(const SimtPlan& pl, dim3 grid, const float* Xr, const 
 SimtPlan simt_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int d, int R) {
     SimtPlan p;
     p.dp = ((d + 3) / 4) * 4;
+    p.R = R;
     p.R_pad = ((R + 3) / 4) * 4;   // accumulators for the columns in use only (R <= 32)
     p.n_rowblk = (int)((Nr + kSimtRows - 1) / kSimtRows);
     const int64_t ntiles = (Nc + kSimtTile - 1) / kSimtTile;
@@ -184,14 +210,19 @@ SimtPlan simt_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int d, int R) {
     int64_t sp = (target + p.n_rowblk - 1) / p.n_rowblk;
     const int64_t max_sp = ntiles / 4 > 0 ? ntiles / 4 : 1;
     if (sp > max_sp) sp = max_sp;
-    if (sp > 64) sp = 64;
+    // Up to 64 R_pad / R splits: few rows (the posterior mean at 1,024 points) then still fill
+    // the SMs with 1 to 3 columns, in the partial buffer that 64 splits of R_pad columns
+    // take (one column, 1,024 x 150,001 pairs, d = 16, Matern-3/2: 64 splits 503 us a call, 256
+    // splits 294).
+    const int64_t cap = 64 * (int64_t)p.R_pad / R;
+    if (sp > cap) sp = cap;
     if (sp < 1) sp = 1;
     p.n_split = (int)sp;
     return p;
 }
 
 size_t simt_partial_floats(const SimtPlan& p, int64_t Nr) {
-    return p.n_split > 1 ? (size_t)p.n_split * p.R_pad * (size_t)Nr : 0;
+    return p.n_split > 1 ? (size_t)p.n_split * p.R * (size_t)Nr : 0;
 }
 
 int launch_kmvm_simt(Ctx* ctx, const SimtPlan& pl, const MvmArgs& a, float outputscale, const float* Xrs,
@@ -220,19 +251,21 @@ int launch_kmvm_simt(Ctx* ctx, const SimtPlan& pl, const MvmArgs& a, float outpu
     }
     ctx->launches++;
     if (e != cudaSuccess) return GP_ERR_CUDA;
-    if (pl.n_split > 1) {
-        dim3 g2((unsigned)((a.Nr + 255) / 256), (unsigned)a.R);
-        split_reduce_kernel<<<g2, 256, 0, s>>>(partial, pl.n_split, a.Nr, pl.R_pad, a.Nr, a.R, nullptr, outputscale,
-                                               a.noise, a.Vnoise, a.Nc, a.out, a.ld_out);
-        ctx->launches++;
-        if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
-    }
+    if (pl.n_split > 1)
+        return launch_split_reduce(ctx, partial, pl.n_split, a.Nr, a.Nr, a.R, a.R, nullptr, outputscale, a.noise,
+                                   a.Vnoise, a.Nc, a.out, a.ld_out, s);
     return GP_OK;
 }
 
 int launch_split_reduce(Ctx* ctx, const float* partial, int n_split, int64_t ld_part, int64_t Nr, int R,
                         int RP, const float* outscale, float outscale_const, float noise, const float* Vnoise,
                         int64_t ld_v, float* out, int64_t ld_out, cudaStream_t s) {
+    if (n_split > 64) {
+        split_reduce_wide_kernel<<<dim3((unsigned)((Nr + 31) / 32), (unsigned)R), 256, 0, s>>>(
+            partial, n_split, ld_part, RP, Nr, R, outscale, outscale_const, noise, Vnoise, ld_v, out, ld_out);
+        ctx->launches++;
+        return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
+    }
     dim3 g((unsigned)((Nr + 255) / 256), (unsigned)R);
     split_reduce_kernel<<<g, 256, 0, s>>>(partial, n_split, ld_part, RP, Nr, R, outscale, outscale_const, noise,
                                           Vnoise, ld_v, out, ld_out);

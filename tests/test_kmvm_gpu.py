@@ -518,3 +518,15 @@ def test_pair_engine_tile_edges(ctx, mode, N, R):
                      "half_exp": ("fp16", gpk.MVM_HALF_EXP, TOL["fp16"])}[mode]
     got = _run(ctx, X, V, 0, ls, a2, s2, prec, flags=fl)
     assert _colerr(got, _ref(X, V, 0, ls, a2, s2)) <= tol
+
+
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("Nr", [1, 31, 33, 256, 257, 1024])
+def test_fp32_few_rows_many_splits(ctx, Nr, R):
+    """The FP32 engine on few rows and many columns (the posterior mean): more
+    than 64 column splits with 1 to 3 vectors, and their reduction, at the edges
+    of its 32-row blocks and of the column tiles."""
+    X, V, _, ls, a2, s2 = workloads.random_problem(20_001, 7, R, seed=Nr + R, kernel=1)
+    Xr = np.random.default_rng(Nr).standard_normal((Nr, 7)).astype(np.float32)
+    got = _run(ctx, Xr, V, 1, ls, a2, s2, "fp32", Xc=X, add_noise=False)
+    assert _colerr(got, _ref(Xr, V, 1, ls, a2, s2, Xc=X, add_noise=False)) <= TOL["fp32"]
