@@ -9,10 +9,18 @@
 // in FP32.  One launch per step: every block first reduces the previous
 // step's per-block argmax candidates (a few hundred pairs), so no separate
 // global argmax pass is needed; the kernel row is evaluated on the fly from
-// the scaled inputs (SIMT FP32, same kernel forms as the MVM).
+// the scaled inputs (SIMT FP32, same kernel forms as the MVM).  A step is a chain
+// of latencies (launch, candidates, pivot row, the earlier columns, argmax), so
+// the launches overlap (programmatic dependent launch) and the earlier columns are
+// loaded sixteen at a time (the whole factor and core at N = 65,536, d = 8, rank 100:
+// 1.51 -> 0.95 ms a call; the core's 530 us and the inverse's 254 us are what the lines
+// below took away).
 //
 // Core.  C = I + sigma^-2 L^T L is accumulated in FP64 from FP32 sums of
-// 64-row chunks and factored C = Lc Lc^T in FP64 by one CTA.
+// 64-row chunks, its lower triangle only, and factored C = Lc Lc^T in FP64 by
+// one CTA.  FP64 runs at two multiply-adds per cycle and SM here, so the sums
+// over the row splits are spread over the SMs and the factorisation keeps
+// square roots and divisions off its chain (one reciprocal per column).
 //
 // Apply.  P^{-1} w = sigma^-2 w - sigma^-4 L C^{-1} L^T w: t = L^T w (FP32
 // within 256-row blocks, FP64 across blocks, fixed order), u = C^{-1} t by
@@ -72,8 +80,10 @@ __global__ void __launch_bounds__(kPcThreads)
 pivchol_step_kernel(const float* __restrict__ Xs, int64_t N, int dp, int m, float a2, float tol_abs,
                     float* __restrict__ L, float* __restrict__ diag, const Cand* __restrict__ cin, int g_in,
                     Cand* __restrict__ cout, int* __restrict__ piv, int* __restrict__ rank_out) {
-    __shared__ float sxp[64];
+    __shared__ __align__(16) float sxp[64];
     __shared__ float slp[512];
+    // launched while the previous step runs (programmatic dependent launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (*rank_out >= 0) return;   // an earlier step stopped the factorisation
     float dmax;
     int p;
@@ -98,17 +108,36 @@ pivchol_step_kernel(const float* __restrict__ Xs, int64_t N, int dp, int m, floa
     for (int q = threadIdx.x; q < m; q += blockDim.x) slp[q] = L[(int64_t)q * N + p];
     __syncthreads();
     const float inv = 1.0f / sqrtf(dmax);
+    const float4* xp4 = reinterpret_cast<const float4*>(sxp);
     float bv = -INFINITY;
     int bi = 0x7fffffff;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         float q2 = 0.0f;
-        for (int k = 0; k < dp; ++k) {
-            const float df = Xs[i * dp + k] - sxp[k];
+        const float4* x4 = reinterpret_cast<const float4*>(Xs + i * dp);   // dp is a multiple of 4
+        for (int k = 0; k < dp / 4; ++k) {
+            const float4 a = x4[k], b = xp4[k];
+            float df = a.x - b.x;
+            q2 = fmaf(df, df, q2);
+            df = a.y - b.y;
+            q2 = fmaf(df, df, q2);
+            df = a.z - b.z;
+            q2 = fmaf(df, df, q2);
+            df = a.w - b.w;
             q2 = fmaf(df, df, q2);
         }
         const float kv = a2 * kernel_from_s<KIND>(-q2);
         float dot = 0.0f;
-        for (int q = 0; q < m; ++q) dot = fmaf(L[(int64_t)q * N + i], slp[q], dot);
+        const float* li = L + i;
+        int q = 0;
+        for (; q + 16 <= m; q += 16) {   // sixteen loads in flight, the same order of additions
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = li[(int64_t)(q + u) * N];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) dot = fmaf(v[u], slp[q + u], dot);
+        }
+#pragma unroll 4
+        for (; q < m; ++q) dot = fmaf(li[(int64_t)q * N], slp[q], dot);
         const float lv = (kv - dot) * inv;
         L[(int64_t)m * N + i] = lv;
         const float dn = (i == p) ? 0.0f : diag[i] - lv * lv;
@@ -124,70 +153,118 @@ __global__ void fill_kernel(float* p, int64_t n, float v) {
         p[i] = v;
 }
 
-// partial[s][a][b] = sum over rows of split s of L[a][i] L[b][i], FP64.
-// grid = (tiles of 16 x 16 over k x k, splits); L column-major (ld N).
-__global__ void gram_ll_kernel(const float* __restrict__ L, int64_t N, int k, int nsplit,
-                               double* __restrict__ partial) {
-    __shared__ float sa[64][17];
-    __shared__ float sb[64][17];
-    const int tiles = (k + 15) / 16;
-    const int ta = blockIdx.x / tiles, tb = blockIdx.x % tiles;
+// partial[s][a][b] = sum over rows of split s of L[a][i] L[b][i], FP64, for the
+// 32 x 32 tiles with a >= b's tile (C is symmetric, products commute exactly).
+// grid = (lower tiles, splits); L column-major (ld N); 2 x 2 entries per thread.
+constexpr int kGramTile = 32;
+__global__ void __launch_bounds__(256)
+gram_ll_kernel(const float* __restrict__ L, int64_t N, int k, int nsplit, double* __restrict__ partial) {
+    __shared__ float sa[64][kGramTile + 2];
+    __shared__ float sb[64][kGramTile + 2];
+    int ta = 0, t = blockIdx.x;
+    while (t > ta) { t -= ta + 1; ++ta; }   // lower tile (ta, tb), tb <= ta
+    const int tb = t;
     const int s = blockIdx.y;
-    const int la = threadIdx.x >> 4, lb = threadIdx.x & 15;   // 256 threads: 16 x 16
-    const int a = ta * 16 + la, b = tb * 16 + lb;
+    const int la = (threadIdx.x >> 4) * 2, lb = (threadIdx.x & 15) * 2;   // 16 x 16 threads
     const int64_t r0 = (N * s) / nsplit, r1 = (N * (s + 1)) / nsplit;
-    double acc = 0.0;
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
     for (int64_t i0 = r0; i0 < r1; i0 += 64) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            const int ii = e % 64, cc = e / 64;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = threadIdx.x + q * 256, ii = e & 63, cc = e >> 6;
             const int64_t i = i0 + ii;
-            const int ca = ta * 16 + cc, cb = tb * 16 + cc;
+            const int ca = ta * kGramTile + cc, cb = tb * kGramTile + cc;
             sa[ii][cc] = (i < r1 && ca < k) ? L[(int64_t)ca * N + i] : 0.0f;
             sb[ii][cc] = (i < r1 && cb < k) ? L[(int64_t)cb * N + i] : 0.0f;
         }
         __syncthreads();
         // 64 products in FP32, the chunk sums in FP64 (FP64 is scarce on this GPU)
-        float cs = 0.0f;
+        float cs[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll 16
-        for (int ii = 0; ii < 64; ++ii) cs = fmaf(sa[ii][la], sb[ii][lb], cs);
-        acc += (double)cs;
+        for (int ii = 0; ii < 64; ++ii) {
+            const float2 va = *reinterpret_cast<const float2*>(&sa[ii][la]);
+            const float2 vb = *reinterpret_cast<const float2*>(&sb[ii][lb]);
+            cs[0][0] = fmaf(va.x, vb.x, cs[0][0]);
+            cs[0][1] = fmaf(va.x, vb.y, cs[0][1]);
+            cs[1][0] = fmaf(va.y, vb.x, cs[1][0]);
+            cs[1][1] = fmaf(va.y, vb.y, cs[1][1]);
+        }
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int y = 0; y < 2; ++y) acc[x][y] += (double)cs[x][y];
         __syncthreads();
     }
-    if (a < k && b < k) partial[((int64_t)s * k + a) * k + b] = acc;
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const int a = ta * kGramTile + la + x, b = tb * kGramTile + lb + y;
+            if (a < k && b < k) partial[((int64_t)s * k + a) * k + b] = acc[x][y];
+        }
 }
 
-// One CTA: C = I + sigma^-2 sum_s partial[s], then in-place FP64 Cholesky.
-// core (k x k, column-major) receives the lower factor (upper part zeroed).
-__global__ void core_chol_kernel(const double* __restrict__ partial, int nsplit, int k, double inv_noise,
-                                 double* __restrict__ core, int* err) {
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-        const int a = e % k, b = e / k;   // row a, column b
-        double g = 0.0;
+// core(a, b) = (a == b) + sigma^-2 sum_s partial[s][a][b] for a >= b (column-major
+// lower triangle, upper zeroed); one thread per entry, splits in order.
+__global__ void core_sum_kernel(const double* __restrict__ partial, int nsplit, int k, double inv_noise,
+                                double* __restrict__ core) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= k * k) return;
+    const int a = e / k, b = e % k;   // row a, column b: b fastest in partial
+    double g = 0.0;
+    if (a >= b) {
+#pragma unroll 8
         for (int s = 0; s < nsplit; ++s) g += partial[((int64_t)s * k + a) * k + b];
-        core[(int64_t)b * k + a] = (a == b ? 1.0 : 0.0) + inv_noise * g;
+        g = (a == b ? 1.0 : 0.0) + inv_noise * g;
+    }
+    core[(int64_t)b * k + a] = g;
+}
+
+// One CTA: in-place FP64 Cholesky of the lower triangle in core (k x k,
+// column-major).  The elimination runs as L D L^T (column j updates the rest
+// with l_ij l_lj / d_j: one reciprocal per column) and the columns are
+// scaled by 1 / sqrt(d_j) at the end.  In shared memory when the triangle fits.
+__global__ void __launch_bounds__(512)
+core_chol_kernel(int k, int in_smem, double* __restrict__ core, int* err) {
+    extern __shared__ double smem[];   // w [k], then the matrix (in_smem)
+    double* w = smem;
+    double* A = core;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (in_smem) {
+        A = smem + k;
+        for (int e = tid; e < k * k; e += nt) A[e] = core[e];
     }
     __syncthreads();
-    __shared__ double piv;
     for (int j = 0; j < k; ++j) {
-        if (threadIdx.x == 0) {
-            const double djj = core[(int64_t)j * k + j];
-            if (!(djj > 0.0)) atomicCAS(err, 0, (int)DEV_BREAKDOWN);
-            piv = sqrt(djj > 0.0 ? djj : 1.0);
-            core[(int64_t)j * k + j] = piv;
+        const double* cj = A + (int64_t)j * k;
+        if (tid < 32) {   // one warp: w_l = l_lj / d_j
+            double d = cj[j];
+            if (!(d > 0.0)) {
+                if (tid == 0) atomicCAS(err, 0, (int)DEV_BREAKDOWN);
+                d = 1.0;
+            }
+            const double r = 1.0 / d;
+            for (int l = j + 1 + tid; l < k; l += 32) w[l] = cj[l] * r;
         }
         __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < k; i += blockDim.x) core[(int64_t)j * k + i] /= piv;
-        __syncthreads();
-        const int rem = k - j - 1;
-        for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-            const int i = j + 1 + e % rem, l = j + 1 + e / rem;
-            if (l <= i) core[(int64_t)l * k + i] -= core[(int64_t)j * k + i] * core[(int64_t)j * k + l];
+        // warps take columns l of the remaining triangle, lanes its rows i >= l
+        for (int l = j + 1 + (tid >> 5); l < k; l += nt >> 5) {
+            double* cl = A + (int64_t)l * k;
+            const double wl = w[l];
+            for (int i = l + (tid & 31); i < k; i += 32) cl[i] = fma(-cj[i], wl, cl[i]);
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-        const int a = e % k, b = e / k;
-        if (a < b) core[(int64_t)b * k + a] = 0.0;
+    for (int j = tid; j < k; j += nt) {
+        const double d = A[(int64_t)j * k + j];
+        w[j] = 1.0 / sqrt(d > 0.0 ? d : 1.0);
+    }
+    __syncthreads();
+    for (int e = tid; e < k * k; e += nt) {
+        const int i = e % k, j = e / k;
+        if (i < j) continue;
+        const double d = A[e];
+        core[e] = (i == j) ? (d > 0.0 ? d : 1.0) * w[j] : d * w[j];
     }
 }
 
@@ -199,44 +276,54 @@ __global__ void core_chol_kernel(const double* __restrict__ partial, int nsplit,
 // them), u = C^{-1} t (one warp per output), z = (w - L u / sigma^2) / sigma^2.
 
 // Column j of C^{-1} = Lc^{-T} Lc^{-1} e_j: forward and backward substitution,
-// one warp per column, lane l holding rows l + 32 m (k <= 32 PER).
-// Lc is column-major: Lc(a, b) = core[b * k + a].
+// both column-oriented (one multiplication by the stored reciprocal of the
+// diagonal, one shuffle and one FMA per step of the chain), one warp per
+// column, lane l holding rows l + 32 m (k <= 32 PER).  Lc is column-major:
+// Lc(a, b) = core[b * k + a], staged in shared memory when it fits (in_smem).
 template <int PER>
-__global__ void __launch_bounds__(256)
-core_inverse_kernel(const double* __restrict__ core, int k, double* __restrict__ cinv) {
-    const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(128)
+core_inverse_kernel(const double* __restrict__ core, int k, int in_smem, double* __restrict__ cinv) {
+    extern __shared__ double smem[];   // reciprocals [k], then the factor (in_smem)
+    double* rd = smem;
+    const double* A = core;
+    if (in_smem) {
+        double* sA = smem + k;
+        for (int e = threadIdx.x; e < k * k; e += blockDim.x) sA[e] = core[e];
+        A = sA;
+    }
+    for (int a = threadIdx.x; a < k; a += blockDim.x) rd[a] = 1.0 / core[(int64_t)a * k + a];
+    __syncthreads();
+    const int j = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= k) return;
     double y[PER];
 #pragma unroll
     for (int m = 0; m < PER; ++m) y[m] = (lane + 32 * m == j) ? 1.0 : 0.0;
-    // forward, column-oriented (entries above j stay zero)
-    for (int a = j; a < k; ++a) {
-        const double* col = core + (int64_t)a * k;
-        double ya = 0.0;
+    // forward (entries above j stay zero); the blocks of 32 rows are unrolled so that y stays in registers
 #pragma unroll
-        for (int m = 0; m < PER; ++m)
-            if (lane + 32 * m == a) ya = y[m] / col[a];
-        ya = __shfl_sync(0xffffffffu, ya, a & 31);
+    for (int q = 0; q < PER; ++q) {
+        for (int a = (j > 32 * q ? j : 32 * q); a < 32 * q + 32 && a < k; ++a) {
+            const double* col = A + (int64_t)a * k;
+            const double ya = __shfl_sync(0xffffffffu, y[q], a & 31) * rd[a];
 #pragma unroll
-        for (int m = 0; m < PER; ++m) {
-            const int i = lane + 32 * m;
-            if (i == a) y[m] = ya;
-            else if (i > a && i < k) y[m] = fma(-col[i], ya, y[m]);
+            for (int m = q; m < PER; ++m) {
+                const int i = lane + 32 * m;
+                if (i == a) y[m] = ya;
+                else if (i > a && i < k) y[m] = fma(-col[i], ya, y[m]);
+            }
         }
     }
-    // backward, row-oriented: x_a = (y_a - sum_{i > a} Lc(i, a) x_i) / Lc(a, a)
-    for (int a = k - 1; a >= 0; --a) {
-        const double* col = core + (int64_t)a * k;
-        double sacc = 0.0;
+    // backward: x_a, then y_i -= Lc(a, i) x_a for i < a
 #pragma unroll
-        for (int m = 0; m < PER; ++m) {
-            const int i = lane + 32 * m;
-            if (i > a && i < k) sacc = fma(col[i], y[m], sacc);
+    for (int q = PER - 1; q >= 0; --q) {
+        for (int a = (k - 1 < 32 * q + 31 ? k - 1 : 32 * q + 31); a >= 32 * q; --a) {
+            const double ya = __shfl_sync(0xffffffffu, y[q], a & 31) * rd[a];
+#pragma unroll
+            for (int m = 0; m <= q; ++m) {
+                const int i = lane + 32 * m;
+                if (i == a) y[m] = ya;
+                else if (i < a) y[m] = fma(-A[(int64_t)i * k + a], ya, y[m]);
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
-#pragma unroll
-        for (int m = 0; m < PER; ++m)
-            if (lane + 32 * m == a) y[m] = (y[m] - sacc) / col[a];
     }
 #pragma unroll
     for (int m = 0; m < PER; ++m) {
@@ -429,6 +516,12 @@ size_t pivchol_workspace(const Ctx* ctx, int64_t N, int d, int rank) {
     return c.off;
 }
 
+namespace {
+// Shared memory of the one-CTA core kernels: a vector, and the k x k matrix when it fits 200 KB (k <= 159).
+int core_in_smem(int k) { return (size_t)(k + 1) * k * sizeof(double) <= 200 * 1024 ? 1 : 0; }
+size_t core_smem(int k) { return (size_t)(core_in_smem(k) ? (k + 1) * k : k) * sizeof(double); }
+}  // namespace
+
 int pivchol_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int64_t N, int rank, float* L,
                 int32_t* piv, double* core, int* rank_out_host, cudaStream_t s) {
     const int dp = ((hyp->d + 3) / 4) * 4;
@@ -455,27 +548,25 @@ int pivchol_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int
     if (!rank_out_host && cudaMemsetAsync(L, 0, sizeof(float) * (size_t)N * rank, s) != cudaSuccess)
         return GP_ERR_CUDA;
     const float tol_abs = 1e-6f * a2;
+    auto step = hyp->kernel == GP_KERNEL_RBF        ? pivchol_step_kernel<GP_KERNEL_RBF>
+                : hyp->kernel == GP_KERNEL_MATERN32 ? pivchol_step_kernel<GP_KERNEL_MATERN32>
+                : hyp->kernel == GP_KERNEL_MATERN12 ? pivchol_step_kernel<GP_KERNEL_MATERN12>
+                                                    : pivchol_step_kernel<GP_KERNEL_MATERN52>;
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)G);
+    cfg.blockDim = dim3(kPcThreads);
+    cfg.stream = s;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = 1;
     for (int m = 0; m < rank; ++m) {
         const Cand* cin = (m & 1) ? ca : cb;
         Cand* cout = (m & 1) ? cb : ca;
-        switch (hyp->kernel) {
-            case GP_KERNEL_RBF:
-                pivchol_step_kernel<GP_KERNEL_RBF><<<G, kPcThreads, 0, s>>>(Xs, N, dp, m, a2, tol_abs, L, diag, cin, G,
-                                                                            cout, piv, rk);
-                break;
-            case GP_KERNEL_MATERN32:
-                pivchol_step_kernel<GP_KERNEL_MATERN32><<<G, kPcThreads, 0, s>>>(Xs, N, dp, m, a2, tol_abs, L, diag,
-                                                                                 cin, G, cout, piv, rk);
-                break;
-            case GP_KERNEL_MATERN12:
-                pivchol_step_kernel<GP_KERNEL_MATERN12><<<G, kPcThreads, 0, s>>>(Xs, N, dp, m, a2, tol_abs, L, diag,
-                                                                                 cin, G, cout, piv, rk);
-                break;
-            default:
-                pivchol_step_kernel<GP_KERNEL_MATERN52><<<G, kPcThreads, 0, s>>>(Xs, N, dp, m, a2, tol_abs, L, diag,
-                                                                                 cin, G, cout, piv, rk);
-                break;
-        }
+        if (cudaLaunchKernelEx(&cfg, step, (const float*)Xs, N, dp, m, a2, tol_abs, L, diag, cin, G, cout, (int*)piv, rk) !=
+            cudaSuccess)
+            return GP_ERR_CUDA;
         ctx->launches++;
     }
     if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
@@ -489,11 +580,16 @@ int pivchol_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int
         *rank_out_host = kr;
     }
     if (kr == 0) return GP_OK;
-    const int tiles = (kr + 15) / 16;
-    gram_ll_kernel<<<dim3(tiles * tiles, nsplit), 256, 0, s>>>(L, N, kr, nsplit, part);
-    ctx->launches++;
-    core_chol_kernel<<<1, 1024, 0, s>>>(part, nsplit, kr, 1.0 / hyp->noise, core, ctx->dev_err);
-    ctx->launches++;
+    const int tiles = (kr + kGramTile - 1) / kGramTile;
+    gram_ll_kernel<<<dim3(tiles * (tiles + 1) / 2, nsplit), 256, 0, s>>>(L, N, kr, nsplit, part);
+    core_sum_kernel<<<(kr * kr + 127) / 128, 128, 0, s>>>(part, nsplit, kr, 1.0 / hyp->noise, core);
+    const int in_smem = core_in_smem(kr);
+    const size_t sh = core_smem(kr);
+    if (sh > 48 * 1024 && cudaFuncSetAttribute(core_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) !=
+                              cudaSuccess)
+        return GP_ERR_CUDA;
+    core_chol_kernel<<<1, 512, sh, s>>>(kr, in_smem, core, ctx->dev_err);
+    ctx->launches += 3;
     return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
 }
 
@@ -524,10 +620,14 @@ size_t woodbury_workspace(const Ctx* ctx, int64_t N, int k, int R) {
 }
 
 int woodbury_prepare(Ctx* ctx, const double* core, int k, double* cinv, cudaStream_t s) {
-    const unsigned g = (unsigned)((k + 7) / 8);
-    if (k <= 128) core_inverse_kernel<4><<<g, 256, 0, s>>>(core, k, cinv);
-    else if (k <= 256) core_inverse_kernel<8><<<g, 256, 0, s>>>(core, k, cinv);
-    else core_inverse_kernel<16><<<g, 256, 0, s>>>(core, k, cinv);
+    const unsigned g = (unsigned)((k + 3) / 4);
+    const int in_smem = core_in_smem(k);
+    const size_t sh = core_smem(k);
+    auto fn = k <= 128 ? core_inverse_kernel<4> : (k <= 256 ? core_inverse_kernel<8> : core_inverse_kernel<16>);
+    if (sh > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) != cudaSuccess)
+        return GP_ERR_CUDA;
+    fn<<<g, 128, sh, s>>>(core, k, in_smem, cinv);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
 }

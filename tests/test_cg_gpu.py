@@ -304,3 +304,30 @@ def test_refine_switch_points(ctx):
     with pytest.raises(gpk.GPKError):
         gpk.cg_solve(ctx, hyp, X, B, pc, precision=split, refine_precision="fp16", refine_resid=0.0, restarts=0,
                      **kw)
+
+
+@pytest.mark.parametrize("rank", [1, 31, 32, 33, 64, 100, 128, 129, 159, 160, 257, 300])
+def test_core_factor_and_inverse_rank_edges(ctx, rank):
+    """The FP64 core at the edges of its kernels (32-wide tiles of L^T L, rows per
+    lane of the inverse, the factor in shared and in global memory).  Core: against
+    I + L^T L / sigma^2 from the returned L; the sums run in FP32 over 64 rows, so
+    each entry errs by at most 64 2^-24 of sum |l_a l_b| (4e-6 with the FP64
+    factorisation's error far below).  Inverse: one CG step on the preconditioned
+    system solves P u = b with the check of the FP64 residual of a converged solve."""
+    from paper_2207_06856_gb300 import gpk
+    X, V, kern, ls, a2, s2 = workloads.random_problem(900, 6, 2, seed=rank, kernel=1)
+    hyp = gpk.Hyper(kern, ls, a2, s2)
+    pc = gpk.pivchol(ctx, hyp, _dev(X), rank)
+    assert pc.rank == rank
+    L = pc.L.cpu().numpy().astype(np.float64)
+    Lc = pc.core.cpu().numpy().T
+    assert np.array_equal(np.triu(Lc, 1), np.zeros_like(Lc))
+    C, bound = L @ L.T / s2, np.abs(L) @ np.abs(L).T / s2
+    assert np.all(np.abs(Lc @ Lc.T - np.eye(rank) - C) <= 4e-6 * bound + 1e-12)
+    U, st, info = gpk.cg_solve(ctx, hyp, _dev(X), _dev(V), pc, tol=1e-4, max_iter=200, precision="fp32")
+    ctx.check()
+    assert st == gpk.GP_OK
+    res = O.relative_residual(X, U.cpu().numpy().T, V.T, O.Hyp("matern32", ls, a2, s2))
+    assert res.max() <= 2e-4
+    _, _, plain = gpk.cg_solve(ctx, hyp, _dev(X), _dev(V), None, tol=1e-4, max_iter=200, precision="fp32")
+    assert info["iters"] <= plain["iters"] + 2     # a wrong inverse would not precondition
