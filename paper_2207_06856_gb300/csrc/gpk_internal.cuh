@@ -106,7 +106,7 @@ struct ScaleVec {
 int launch_prep_x(Ctx* ctx, const OperandLayout& L, const float* X, int64_t N, int64_t N_pad, int d,
                   const ScaleVec& inv, const unsigned* bb, void* XA, void* XB, cudaStream_t s);
 // Per-dimension min / max of X (N x d) as order-preserving integer codes:
-// bb[k] = min, bb[d + k] = max.  Deterministic (atomic min / max).
+// bb[k] = ~min, bb[d + k] = max.  Deterministic (atomic max).
 int launch_bbox(Ctx* ctx, const float* X, int64_t N, int d, unsigned* bb, cudaStream_t s);
 int launch_prep_x_f32(Ctx* ctx, const float* X, int64_t N, int64_t N_pad, int d, int dp, const ScaleVec& inv,
                       float* Xs, cudaStream_t s);

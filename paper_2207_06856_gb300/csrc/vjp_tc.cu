@@ -473,7 +473,7 @@ __global__ void vb_prep_kernel(const float* __restrict__ X, int64_t N, int d, Sc
         const int m = (int)(e / N);
         const int64_t i = e % N;
         if (m < d) {
-            const float centre = 0.5f * (decode_order(bb[m]) + decode_order(bb[d + m]));
+            const float centre = 0.5f * (decode_order(~bb[m]) + decode_order(bb[d + m]));
             Vb[e] = (X[i * d + m] - centre) * il.v[m];
         } else {
             Vb[e] = 1.0f;
@@ -513,14 +513,22 @@ vjp_finish_kernel(const float* __restrict__ part, int n_split, int rv, int64_t N
             }
         }
     }
+    // Warp sums of the 32 values by a transposing butterfly: at distance o each lane
+    // hands over the half of its values whose index differs from its own in bit o,
+    // so 31 FP64 additions replace 32 x 5 (the same tree per value) and lane m ends
+    // with the sum of value m.
     __shared__ double red[8][32];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-    for (int m = 0; m < 32; ++m) {
-        double v = lsum[m];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (l == 0) red[w][m] = v;
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (l & o) != 0;
+#pragma unroll
+        for (int m = 0; m < o; ++m) {
+            const double keep = up ? lsum[m + o] : lsum[m], give = up ? lsum[m] : lsum[m + o];
+            lsum[m] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+    red[w][l] = lsum[0];
     __syncthreads();
     if (threadIdx.x < 32) {
         double t = 0.0;
@@ -529,30 +537,34 @@ vjp_finish_kernel(const float* __restrict__ part, int n_split, int rv, int64_t N
     }
 }
 
-// out[s] = sum_b part[b * stride + s] in block order (one thread per slot)
-__global__ void sum_rows_kernel(const double* __restrict__ part, int nb, int stride, int ns, double* __restrict__ out) {
-    const int s = threadIdx.x;
-    if (s >= ns) return;
+// out[s] = sum_b part[b * stride + s], one warp per slot s (lanes stride over b,
+// then a shuffle tree: a fixed order).
+__global__ void __launch_bounds__(32)
+sum_rows_kernel(const double* __restrict__ part, int nb, int stride, double* __restrict__ out) {
+    const int s = blockIdx.x, l = threadIdx.x;
     double t = 0.0;
-    for (int b = 0; b < nb; ++b) t += part[(int64_t)b * stride + s];
-    out[s] = t;
+#pragma unroll 4
+    for (int b = l; b < nb; b += 32) t += part[(int64_t)b * stride + s];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (l == 0) out[s] = t;
 }
 
-// out[c] = u_c^T w_c in FP64, one block per column, fixed-order tree
-__global__ void coldot2_kernel(const float* __restrict__ U, const float* __restrict__ W, int64_t N,
-                               double* __restrict__ out) {
-    const int c = blockIdx.x;
+// part[c * gridDim.x + blk] = the block's part of u_c^T w_c in FP64 (fixed-order tree)
+__global__ void __launch_bounds__(256)
+coldot2_kernel(const float* __restrict__ U, const float* __restrict__ W, int64_t N, double* __restrict__ part) {
+    const int c = blockIdx.y;
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256)
         acc = fma((double)U[(int64_t)c * N + i], (double)W[(int64_t)c * N + i], acc);
-    __shared__ double r[32];
+    __shared__ double r[8];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) r[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += r[q];
-        out[c] = t;
+        for (int q = 0; q < 8; ++q) t += r[q];
+        part[(int64_t)c * gridDim.x + blockIdx.x] = t;
     }
 }
 
@@ -575,6 +587,8 @@ bool vjp_tc_supported(const gp_hyp_t* hyp, int R) {
 }
 
 namespace {
+
+constexpr int kDotBlocks = 16;   // blocks per column of the sigma^2 dots
 
 struct VjpPlan {
     int n_it, n_jt, n_split, grid, rp, kh, rx, rv;
@@ -626,7 +640,7 @@ void vjp_tc_layout(C& c, const VjpPlan& p, int64_t N, int d, int R) {
     c.template take<double>((size_t)p.grid);              // per-CTA sum H k
     c.template take<double>((size_t)p.nblk_f * 32);       // per-block lengthscale sums
     c.template take<double>(64);                          // sums
-    c.template take<double>((size_t)R);                   // column dots
+    c.template take<double>((size_t)R * kDotBlocks);      // column dots, per block
 }
 
 }  // namespace
@@ -663,7 +677,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     double* hk = wc.take<double>((size_t)pl.grid);
     double* lpart = wc.take<double>((size_t)pl.nblk_f * 32);
     double* sums = wc.take<double>(64);
-    double* dots = wc.take<double>((size_t)R);
+    double* dots = wc.take<double>((size_t)R * kDotBlocks);
     if (!wc.ok) return GP_ERR_WORKSPACE;
 
     // H operands: balanced, globally scaled FP16 copies of [u | w] and [w | u]
@@ -737,16 +751,17 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     const float a2kp = (float)hyp->outputscale * kprime_max(hyp->kernel);
     vjp_finish_kernel<<<(unsigned)pl.nblk_f, 256, 0, s>>>(part, pl.n_split, pl.rv, pl.N_pad, xs, Vb, N, d, tl, a2kp,
                                                           scales, pl.rp, gX_dev, lpart);
-    sum_rows_kernel<<<1, 32, 0, s>>>(lpart, pl.nblk_f, 32, d, sums);
-    sum_rows_kernel<<<1, 32, 0, s>>>(hk, pl.grid, 1, 1, sums + 32);
-    coldot2_kernel<<<R, 256, 0, s>>>(U, W, N, dots);
-    ctx->launches += 4;
+    // sums[0, d): lengthscale sums, sums[32]: sum H k, sums[33]: sum_c u_c^T w_c
+    sum_rows_kernel<<<d, 32, 0, s>>>(lpart, pl.nblk_f, 32, sums);
+    sum_rows_kernel<<<1, 32, 0, s>>>(hk, pl.grid, 1, sums + 32);
+    coldot2_kernel<<<dim3(kDotBlocks, R), 256, 0, s>>>(U, W, N, dots);
+    sum_rows_kernel<<<1, 32, 0, s>>>(dots, R * kDotBlocks, 1, sums + 33);
+    ctx->launches += 5;
     if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
-    double hs[64];
-    double hd[32];
-    float hsc[64];
+    // small read-back through the context's pinned scratch (4 KB)
+    double* hs = reinterpret_cast<double*>(ctx->host_pinned);
+    float* hsc = reinterpret_cast<float*>(hs + 64);
     if (cudaMemcpyAsync(hs, sums, sizeof(double) * 64, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(hd, dots, sizeof(double) * R, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaMemcpyAsync(hsc, scales, sizeof(float) * 64, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return GP_ERR_CUDA;
@@ -754,9 +769,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     // dq/dl_m = -(2 / l_m) sum_i x^_im D_im (F already applied); dq/da^2 = 1/2 sum H k / g^2
     for (int k = 0; k < d; ++k) grad_theta_host[k] = -2.0 / (double)hyp->lengthscale[k] * hs[k];
     grad_theta_host[d] = 0.5 * hs[32] / (g * g);
-    double sg = 0.0;
-    for (int c = 0; c < R; ++c) sg += hd[c];
-    grad_theta_host[d + 1] = sg;
+    grad_theta_host[d + 1] = hs[33];
     return GP_OK;
 }
 
