@@ -147,16 +147,6 @@ struct TpTmem {
     static constexpr uint32_t o(uint32_t w) { return MODE == kWide ? 384u + w * 64u : 128u * NG + w * (256u - 64u * NG); }
 };
 
-__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-// Arrival of an epilogue warp.  A warp whose bounded wait ran out no longer follows
-// the mbarriers, so it waits here instead of running ahead of the barrier's phase.
-__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t threads, bool ok) {
-    if (ok) asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
-    else bar_sync(id, threads);
-}
-
 __device__ __forceinline__ void record_error(int* err, int code) { atomicCAS(err, 0, code); }
 
 __device__ __forceinline__ void item_range(const TpParams& p, int item, int& ip, int& sp, int& j0, int& j1) {
@@ -248,7 +238,7 @@ struct TpSIssue {
     using T = TpTmem<MODE, NG>;
     const TpParams& p;
     TpBarriers& bars;
-    uint32_t aSt, aXi0, xbytes, stage_bytes, arow, hi_x, tmem, id, w;
+    uint32_t aSt, aXi0, xbytes, stage_bytes, arow, hi_x, tmem, id, w, s_full;
     int item, jt, j1, ip, xb;
     uint32_t ic = 0;            // items entered
     uint32_t st = 0, ph = 0;    // stage ring slot and its fill parity
@@ -263,6 +253,7 @@ struct TpSIssue {
         aXi0 = ptx::smem_u32(sXi) + w * xbytes;
         arow = (uint32_t)p.k_pad * 2u;   // 32, 64 or 128 bytes
         hi_x = ptx::smem_desc_hi(8u * arow, (arow == 32) ? 6u : (arow == 64 ? 4u : 2u));
+        s_full = ptx::smem_u32(&bars.s_full[w]);
         item = (int)blockIdx.x - (int)gridDim.x;
         jt = j1 = 0;
     }
@@ -292,13 +283,13 @@ struct TpSIssue {
     // S of columns [h kS, (h + 1) kS) of the selected tile into the ring's next buffer.
     __device__ __forceinline__ void issue(uint32_t h) {
         if (ok) {
-            const uint32_t aXi = aXi0 + (uint32_t)xb * 2u * xbytes, aXj = aSt + st * stage_bytes + h * T::kS * arow;
+            const uint32_t la = ptx::smem_desc_lo(aXi0 + (uint32_t)xb * 2u * xbytes);
+            const uint32_t lb = ptx::smem_desc_lo(aSt + st * stage_bytes + h * T::kS * arow);
+            const uint32_t tD = tmem + T::s(b, w), bar = s_full + 16u * b;
             ptx::tc_fence_after();
-#pragma unroll 1
-            for (uint32_t k = 0; k < arow; k += 32u)   // K-steps of 16 elements
-                ptx::mma_f16_ss_elect(tmem + T::s(b, w), ptx::smem_desc_at(hi_x, aXi + k),
-                                      ptx::smem_desc_at(hi_x, aXj + k), id, k > 0 ? 1u : 0u);
-            ptx::mma_commit_elect(&bars.s_full[2u * b + w]);
+            if (arow == 32u) ptx::mma_f16_ss_elect_commit<1>(tD, la, lb, hi_x, id, bar);
+            else if (arow == 64u) ptx::mma_f16_ss_elect_commit<2>(tD, la, lb, hi_x, id, bar);
+            else ptx::mma_f16_ss_elect_commit<4>(tD, la, lb, hi_x, id, bar);
         }
         if (++b == NG) { b = 0; bph ^= 1u; }
     }
@@ -307,19 +298,21 @@ struct TpSIssue {
     }
 };
 
-// The value product of one slot: O (+)= P Vt^T over 128 (WIDE) or 64 columns.
-template <int MODE, int NG, int PSPLIT>
-__device__ __forceinline__ void tp_value_product(uint32_t tO, uint32_t tP, uint32_t aV, uint32_t kblk, uint32_t id_pv,
-                                                 uint32_t acc) {
-    const uint32_t hi_128 = ptx::smem_desc_hi(1024u, 2u);
-    const uint64_t dV = ptx::smem_desc_at(hi_128, aV);
+// The value product of one slot, O (+)= P Vt^T over 128 (WIDE) or 64 columns, and
+// its commit on `bar`.  lV: descriptor word of Vt, kb: 64-column K-block in 16-byte units.
+template <int MODE, int PSPLIT>
+__device__ __forceinline__ void tp_value_product(uint32_t tO, uint32_t tP, uint32_t lV, uint32_t kb, uint32_t id_pv,
+                                                 uint32_t acc, uint32_t bar) {
+    const uint32_t hi = ptx::smem_desc_hi(1024u, 2u);
     ptx::tc_fence_after();
     if constexpr (MODE == kWide) {
-        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP, dV, id_pv, acc);
-        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP + 32u, ptx::smem_desc_at(hi_128, aV + kblk), id_pv, 1u);
+        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP, lV, hi, id_pv, acc, 0u);
+        ptx::mma_f16_ts4_elect<8, 16, 24>(tO, tP + 32u, lV + kb, hi, id_pv, 1u, bar);
+    } else if constexpr (PSPLIT) {
+        ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP, lV, hi, id_pv, acc, 0u);
+        ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP + 16u, lV, hi, id_pv, 1u, bar);
     } else {
-        ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP, dV, id_pv, acc);
-        if constexpr (PSPLIT) ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP + 16u, dV, id_pv, 1u);
+        ptx::mma_f16_ts4_elect<8, 32, 40>(tO, tP, lV, hi, id_pv, acc, bar);
     }
 }
 
@@ -331,7 +324,8 @@ __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sS
                           uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t id_pv, uint32_t w) {
     using T = TpTmem<MODE, NG>;
     TpSIssue<MODE, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
-    const uint32_t aV0 = ptx::smem_u32(sSt) + xbytes, kblk = (uint32_t)p.rv * 128u;
+    const uint32_t lV0 = ptx::smem_desc_lo(ptx::smem_u32(sSt) + xbytes), kb = (uint32_t)p.rv * 8u;
+    const uint32_t p_empty = ptx::smem_u32(&bars.p_empty[w]);
     const uint32_t tO = tmem + T::o(w);
     uint32_t st = 0, ph = 0, b = 0;
     if constexpr (MODE == kWide) {
@@ -347,27 +341,22 @@ __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sS
 #pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
-            const uint32_t aV = aV0 + st * stage_bytes;
+            const uint32_t lV = lV0 + st * (stage_bytes >> 4);
             if constexpr (MODE == kWide) {
                 // (this tile's stage landed before its S was issued)
-                bar_sync(bar_s_read(w), kBarThreads);
+                ptx::bar_sync(bar_s_read(w), kBarThreads);
                 si.next();
                 if (si.have) { si.issue(0); si.next_stage(); }
-                bar_sync(bar_p_full(w), kBarThreads);
-                if (si.ok) {
-                    tp_value_product<MODE, NG, PSPLIT>(tO, tmem + T::p(0, w), aV, kblk, id_pv, acc);
-                    ptx::mma_commit_elect(&bars.p_empty[w]);
-                }
+                ptx::bar_sync(bar_p_full(w), kBarThreads);
+                if (si.ok) tp_value_product<MODE, PSPLIT>(tO, tmem + T::p(0, w), lV, kb, id_pv, acc, p_empty);
             } else {
                 si.ok = si.ok && warp_wait(&bars.full[st], ph, p.limit_ns);
 #pragma unroll
                 for (uint32_t h = 0; h < 2; ++h) {
-                    bar_sync(bar_p_full(2u * b + w), kBarThreads);
-                    if (si.ok) {
-                        tp_value_product<MODE, NG, PSPLIT>(tO, tmem + T::p(b, w), aV + h * kblk, kblk, id_pv,
-                                                           h > 0 ? 1u : acc);
-                        ptx::mma_commit_elect(&bars.p_empty[2u * b + w]);
-                    }
+                    ptx::bar_sync(bar_p_full(2u * b + w), kBarThreads);
+                    if (si.ok)
+                        tp_value_product<MODE, PSPLIT>(tO, tmem + T::p(b, w), lV + h * kb, kb, id_pv, h > 0 ? 1u : acc,
+                                                       p_empty + 16u * b);
                     if (++b == NG) b = 0;
                 }
             }
@@ -410,16 +399,16 @@ __device__ void tp_issuer_spv(const TpParams& p, TpBarriers& bars, const uint8_t
     TpSIssue<kSpv, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
     uint32_t n = 0;
     for (si.next(); si.have; si.next(), ++n) {
-        if (n >= NG) bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
+        if (n >= NG) ptx::bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
         si.issue(0);
         si.next_stage();
     }
     for (uint32_t q = 0; q < (n < NG ? n : NG); ++q) {   // the epilogue's last reads
         if (n >= NG) {
-            bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
+            ptx::bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
             if (++si.b == NG) si.b = 0;
         } else {
-            bar_sync(bar_s_read(2u * q + w), kBarThreads);
+            ptx::bar_sync(bar_s_read(2u * q + w), kBarThreads);
         }
     }
     ptx::mma_commit_elect(&bars.drain[w]);
@@ -529,7 +518,7 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
                         ptx::tmem_reg_fence(rb);
                     }
                     ptx::tc_fence_before();
-                    bar_arrive(bar_s_read((uint32_t)tl), kBarThreads, ok);   // S is in registers
+                    ptx::bar_arrive(bar_s_read((uint32_t)tl), kBarThreads, ok);   // S is in registers
                     if constexpr (HS) {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) pk[e] = ptx::ex2_h2(ra[e]);
@@ -567,7 +556,7 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
                 }
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before();
-                bar_arrive(bar_p_full(buf), kBarThreads, ok);
+                ptx::bar_arrive(bar_p_full(buf), kBarThreads, ok);
                 if (++b == NG) { b = 0; ph ^= 1u; }
             }
             any = true;
@@ -665,7 +654,7 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
                 ptx::tmem_reg_fence(rr);
                 if (hh == 1) {
                     ptx::tc_fence_before();
-                    bar_arrive(bar_s_read(2u * buf + (uint32_t)tl), kBarThreads, ok);
+                    ptx::bar_arrive(bar_s_read(2u * buf + (uint32_t)tl), kBarThreads, ok);
                 }
 #pragma unroll
                 for (int c4 = 0; c4 < 4; ++c4) {      // 16-byte chunk c: columns [8 c, 8 c + 8) of the 64

@@ -96,6 +96,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
     }
 }
 
+// ---- named barriers (id 0 is __syncthreads) -----------------------------------
+__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// Arrival of a warp that goes on.  A warp whose bounded wait ran out (ok = false) no
+// longer follows the mbarriers, so it waits here instead of running ahead of the
+// barrier's phase.
+__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t threads, bool ok) {
+    if (ok) asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+    else bar_sync(id, threads);
+}
+
 // ---- TMA --------------------------------------------------------------------
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
     asm volatile(
@@ -170,26 +182,85 @@ __device__ __forceinline__ void mma_f16_ts_elect(uint32_t d_tmem, uint32_t a_tme
         "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Four K-steps of the same (64 K-elements): A at TMEM columns 0, A1, A2, A3 from
-// a_tmem, B advancing by 32 bytes inside its 128-byte swizzle atom.  One
-// elect.sync for the four.
+// The issuing warps share their scheduler with four arithmetic warps, where every
+// instruction waits its turn, so the groups below keep the instruction count down: one
+// elect.sync per group, descriptors as a constant high and an advancing low 32-bit word
+// (a group of four in 95 cycles instead of 170 beside busy warps), and the commit of
+// the group inside it (bar: shared-memory address of the mbarrier, 0: no commit).
+
+// Four K-steps of a .ts product (64 K-elements): A at TMEM columns 0, A1, A2, A3
+// from a_tmem, B advancing by 32 bytes inside its 128-byte swizzle atom.
 template <int A1, int A2, int A3>
-__device__ __forceinline__ void mma_f16_ts4_elect(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                                  uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16_ts4_elect(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi,
+                                                  uint32_t idesc, uint32_t accumulate, uint32_t bar) {
     asm volatile(
-        "{\n\t.reg .pred p, t, e;\n\t"
-        ".reg .b32 a1, a2, a3;\n\t"
-        ".reg .b64 b1, b2, b3;\n\t"
+        "{\n\t.reg .pred p, t, e, c;\n\t"
+        ".reg .b32 a1, a2, a3, l1, l2, l3;\n\t"
+        ".reg .b64 b0, b1, b2, b3;\n\t"
         "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 t, %5, 0;\n\t"
-        "add.u32 a1, %1, %6;\n\tadd.u32 a2, %1, %7;\n\tadd.u32 a3, %1, %8;\n\t"
-        "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(1u), "n"(A1), "n"(A2), "n"(A3)
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "setp.eq.b32 t, %0, %0;\n\t"
+        "setp.ne.and.b32 c, %6, 0, e;\n\t"
+        "add.u32 a1, %1, %7;\n\tadd.u32 a2, %1, %8;\n\tadd.u32 a3, %1, %9;\n\t"
+        "add.u32 l1, %2, 2;\n\tadd.u32 l2, %2, 4;\n\tadd.u32 l3, %2, 6;\n\t"
+        "mov.b64 b0, {%2, %3};\n\tmov.b64 b1, {l1, %3};\n\tmov.b64 b2, {l2, %3};\n\tmov.b64 b3, {l3, %3};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b0, %4, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %4, t;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %4, t;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %4, t;\n\t"
+        "@c tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(bar), "n"(A1), "n"(A2), "n"(A3)
+        : "memory");
+}
+// KS = 1, 2 or 4 K-steps of an .ss product, overwriting D: A and B advance by 32
+// bytes inside their swizzle atom (32, 64 or 128 bytes).
+template <int KS>
+__device__ __forceinline__ void mma_f16_ss_elect_commit(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                                        uint32_t idesc, uint32_t bar) {
+    static_assert(KS == 1 || KS == 2 || KS == 4, "");
+    if constexpr (KS == 1) {
+        asm volatile(
+            "{\n\t.reg .pred z, e;\n\t.reg .b64 a0, b0;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 z, %0, %0;\n\t"
+            "mov.b64 a0, {%1, %3};\n\tmov.b64 b0, {%2, %3};\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %4, z;\n\t"
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(bar)
+            : "memory");
+    } else if constexpr (KS == 2) {
+        asm volatile(
+            "{\n\t.reg .pred z, t, e;\n\t.reg .b32 x1, y1;\n\t.reg .b64 a0, b0, a1, b1;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 z, %0, %0;\n\tsetp.eq.b32 t, %0, %0;\n\t"
+            "add.u32 x1, %1, 2;\n\tadd.u32 y1, %2, 2;\n\t"
+            "mov.b64 a0, {%1, %3};\n\tmov.b64 b0, {%2, %3};\n\tmov.b64 a1, {x1, %3};\n\tmov.b64 b1, {y1, %3};\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %4, z;\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %4, t;\n\t"
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(bar)
+            : "memory");
+    } else {
+        asm volatile(
+            "{\n\t.reg .pred z, t, e;\n\t.reg .b32 x1, y1, x2, y2, x3, y3;\n\t"
+            ".reg .b64 a0, b0, a1, b1, a2, b2, a3, b3;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 z, %0, %0;\n\tsetp.eq.b32 t, %0, %0;\n\t"
+            "add.u32 x1, %1, 2;\n\tadd.u32 y1, %2, 2;\n\tadd.u32 x2, %1, 4;\n\tadd.u32 y2, %2, 4;\n\t"
+            "add.u32 x3, %1, 6;\n\tadd.u32 y3, %2, 6;\n\t"
+            "mov.b64 a0, {%1, %3};\n\tmov.b64 b0, {%2, %3};\n\tmov.b64 a1, {x1, %3};\n\tmov.b64 b1, {y1, %3};\n\t"
+            "mov.b64 a2, {x2, %3};\n\tmov.b64 b2, {y2, %3};\n\tmov.b64 a3, {x3, %3};\n\tmov.b64 b3, {y3, %3};\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %4, z;\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %4, t;\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %4, t;\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %4, t;\n\t"
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(bar)
+            : "memory");
+    }
+}
+__device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
@@ -228,6 +299,8 @@ __device__ __forceinline__ uint64_t smem_desc_at(uint32_t hi, uint32_t saddr) {
     const uint32_t lo = ((saddr & 0x3FFFFu) >> 4) | (1u << 16);   // LBO = 16 bytes (unused for K-major swizzled)
     return ((uint64_t)hi << 32) | lo;
 }
+// The low word alone.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
 // Instruction descriptor for kind::f16 with FP32 accumulation, K-major A and B.
 // a_bf16/b_bf16: 0 = FP16, 1 = BF16.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int bf16) {
@@ -313,6 +386,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
         "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
         : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 

@@ -23,14 +23,27 @@
 //   H  = UW_i WU_j^T     UW = [a_c u | w / a_c], WU = [w / a_c | a_c u] in FP16
 //                        (a_c a power of two balancing the column pair; one
 //                        global power-of-two scale keeps |entries| <= 1)
-//   O += W'_i Xt_j^T     W' from TMEM (.ts form), Xt = [x^ hi; 1; x^ lo; 0]
-//                        rows (the ones row gives rs_i); N = 2 R_pad
-// The epilogue stores W' / (a^2 k'_max) = -phi(s) H (phi = k for RBF, e^-u for
-// Matern-3/2, (1 + u) e^-u for Matern-5/2) as FP16 in TMEM, and accumulates
-// sum H k per thread.  Warps: 0-15 epilogue (warpgroup q: columns
-// [32 q, 32 q + 32) of the tile), 16 TMA producer, 17 S / H issuer and TMEM
-// owner, 18 value-product issuer.  TMEM: S [0,128), H [128,256), W' buffers
-// [256,320) and [320,384), O [384, 384 + 2 R_pad).  Every wait is bounded.
+//   O += W'_i Xt_j^T     Xt = [x^ hi; 1; x^ lo; 0] rows (the ones row gives rs_i);
+//                        N = rv = 16 ceil(2 (d + 1) / 16)
+// The epilogue forms W' / (a^2 k'_max) = -phi(s) H (phi = k for RBF, e^-u for
+// Matern-3/2, (1 + u) e^-u for Matern-5/2) as FP16 and accumulates sum H k per
+// thread.  A slot is 64 columns of a tile: S and H take 64 TMEM columns each, W' is
+// written over S in place, and three slots form a ring, so that S and H of the next
+// slots and the value product of the last one run behind the epilogue's arithmetic
+// (with one 128-column S and H for all sixteen warps the tensor pipe was 43 % active).
+// The row tile's operands sit in TMEM too (.ts form; copied from shared memory once
+// per item), so a 64-column S or H instruction reads 2 KB of shared memory instead
+// of 6 KB and takes 34 cycles instead of 51.
+//
+// Warps: 0-15 epilogue (warpgroup g: slot parity g & 1, half g >> 1 of its columns),
+// 16 TMA producer, 17 S issuer and TMEM owner, 18 H issuer, 19 value-product issuer;
+// the epilogue tells the issuers by named barriers (see kmvm_tp.cu).  TMEM: slot b S at
+// 128 b, H at 128 b + 64; O at 384; XA_i at 448, UW_i at 480.  Every wait is bounded.
+//
+// N = 65,536, d = 18 (k_pad 64), 17 columns, RBF: 1.58 ms per launch with one
+// 128-column S and H for all warps, 1.18 ms now, against 0.63 of tensor work (760 cycles a
+// tile; ex2 takes 512).  What is left is latency: beside four busy warps an issuer's
+// instruction waits its turn, and a slot passes S / H, epilogue and value product in sequence.
 #include "gpk_internal.cuh"
 #include "ptx.cuh"
 #include "kfun.cuh"
@@ -44,39 +57,17 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kBN = 128;
 constexpr int kEpiWarps = 16;
-constexpr int kThreads = (kEpiWarps + 3) * 32;
+constexpr int kThreads = (kEpiWarps + 4) * 32;
 constexpr int kTmaWarp = kEpiWarps;
-constexpr int kShWarp = kEpiWarps + 1;
-constexpr int kOWarp = kEpiWarps + 2;
+constexpr int kShWarp = kEpiWarps + 1;    // S issuer (TMEM owner), then the H issuer
+constexpr int kOWarp = kEpiWarps + 3;
 constexpr int kMaxStages = 4;
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColS = 0, kColH = 128, kColW = 256, kColO = 384;
+constexpr uint32_t kRing = 3;             // slots of 64 columns
+constexpr uint32_t kColO = 384, kColXA = 448, kColUW = 480;
+constexpr uint32_t kBarThreads = 9 * 32;  // 8 epilogue warps and one issuer (kBarA: two)
+constexpr uint32_t kBarA = 1, kBarW = 2;  // row operands in TMEM; W' of slot b stored (kBarW + b)
 constexpr int kMaxSmemBytes = 227 * 1024;
-
-struct VjpParams {
-    int n_it, n_jt, n_split, n_items;
-    int k_pad, kh, rv;       // S contraction width, H contraction width (2 R_pad), O width (2 R_pad of Xt)
-    int stages;
-    int64_t N_pad;
-    float* part;             // [n_split][rv][N_pad]: raw O columns
-    double* hk;              // [gridDim.x]: per-CTA sum of H k
-    int* err;
-    uint64_t limit_ns;
-};
-
-struct VjpBarriers {
-    uint64_t full[kMaxStages];
-    uint64_t empty[kMaxStages];
-    uint64_t xi_full[2];
-    uint64_t xi_empty[2];
-    uint64_t sh_full;
-    uint64_t sh_empty;
-    uint64_t w_full[2];
-    uint64_t w_empty[2];
-    uint64_t o_full;
-    uint64_t o_empty;
-    uint64_t drain[2];
-};
 
 struct VjpSmem {
     uint32_t xbytes, hbytes, vbytes, stage_bytes, xi_bytes;
@@ -99,13 +90,39 @@ __host__ __device__ inline VjpSmem vjp_smem(int k_pad, int kh, int rv) {
     return m;
 }
 
+struct VjpParams {
+    int n_it, n_jt, n_split, n_items;
+    int k_pad, kh, rv;       // S contraction width, H contraction width (2 R_pad), O width
+    int stages;
+    VjpSmem sm;
+    int64_t N_pad;
+    float* part;             // [n_split][rv][N_pad]: raw O columns
+    double* hk;              // [gridDim.x]: per-CTA sum of H k
+    int* err;
+    uint64_t limit_ns;
+};
+
+struct VjpBarriers {
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
+    uint64_t xi_full[2];
+    uint64_t xi_empty[2];
+    uint64_t sh_full[kRing];
+    uint64_t w_empty[kRing];    // W' consumed: S and H of a later slot may overwrite the buffer
+    uint64_t o_full;
+    uint64_t o_empty;
+    uint64_t drain[3];
+};
+
 __device__ __forceinline__ void record_error(int* err, int code) { atomicCAS(err, 0, code); }
 
 __device__ __forceinline__ void item_range(const VjpParams& p, int item, int& it, int& sp, int& j0, int& j1) {
-    it = item % p.n_it;
-    sp = item / p.n_it;
-    j0 = (int)(((int64_t)sp * p.n_jt) / p.n_split);
-    j1 = (int)(((int64_t)(sp + 1) * p.n_jt) / p.n_split);
+    // 32-bit: n_split <= 16 and n_jt <= 2^24
+    const uint32_t q = (uint32_t)item / (uint32_t)p.n_it;
+    sp = (int)q;
+    it = item - sp * p.n_it;
+    j0 = (int)(q * (uint32_t)p.n_jt / (uint32_t)p.n_split);
+    j1 = (int)((q + 1u) * (uint32_t)p.n_jt / (uint32_t)p.n_split);
 }
 
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
@@ -125,6 +142,7 @@ __device__ void vjp_producer(const VjpParams& p, const CUtensorMap* tmA, const C
     int ic = 0;
     const uint32_t S = (uint32_t)p.stages;
     const uint32_t vbox = (uint32_t)p.rv * 128u;
+#pragma unroll 1
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int it, sp, j0, j1;
         item_range(p, item, it, sp, j0, j1);
@@ -135,9 +153,10 @@ __device__ void vjp_producer(const VjpParams& p, const CUtensorMap* tmA, const C
         ptx::tma_load_2d(sX, tmA, &bars.xi_full[xb], 0, it * kBM);
         ptx::tma_load_2d(sX + m.xbytes, tmUW, &bars.xi_full[xb], 0, it * kBM);
         ++xi_loads;
+#pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             const uint32_t st = fills % S, u = fills / S;
-            if (u > 0 && !ptx::mbar_wait(&bars.empty[st], (u - 1) & 1, p.limit_ns)) { ok = false; break; }
+            if (u > 0 && !ptx::mbar_wait_sleep(&bars.empty[st], (u - 1) & 1, p.limit_ns)) { ok = false; break; }
             uint8_t* sx = sSt + st * m.stage_bytes;
             ptx::mbar_arrive_expect_tx(&bars.full[st], m.stage_bytes);
             ptx::tma_load_2d(sx, tmB, &bars.full[st], 0, jt * kBN);
@@ -158,89 +177,104 @@ __device__ void vjp_producer(const VjpParams& p, const CUtensorMap* tmA, const C
     }
 }
 
-// ---- S / H issuer (one converged warp) ------------------------------------------
-// For each column tile: S and H into their TMEM buffers once the epilogue has
-// read the previous tile's S and H and the stage has landed.
-__device__ void vjp_mma_sh(const VjpParams& p, VjpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
-                           const VjpSmem& m, uint32_t tmem) {
-    const uint32_t xrow = (uint32_t)p.k_pad * 2u, hrow = (uint32_t)p.kh * 2u;
-    const uint32_t hi_x = ptx::smem_desc_hi(8u * xrow, swz_code(xrow));
-    const uint32_t hi_h = ptx::smem_desc_hi(8u * hrow, swz_code(hrow));
-    const uint32_t id = ptx::idesc_f16(kBM, kBN, 0);
-    const uint32_t S = (uint32_t)p.stages;
-    const uint32_t aSt = ptx::smem_u32(sSt);
-    uint32_t g = 0, st = 0, ph = 0;
-    int ic = 0;
+// ---- S and H issuers (two converged warps) ----------------------------------------
+// K-steps of 16 of a 64-column product and its commit: A from TMEM, B rows of
+// `row` bytes (32, 64 or 128) at descriptor word lB.
+__device__ __forceinline__ void vjp_product(uint32_t tD, uint32_t tA, uint32_t lB, uint32_t row, uint32_t hi, uint32_t id,
+                                            uint32_t bar) {
+    if (row == 128u) {
+        ptx::mma_f16_ts4_elect<8, 16, 24>(tD, tA, lB, hi, id, 0u, bar);
+    } else {
+#pragma unroll 1
+        for (uint32_t k = 0; k < row; k += 32u)
+            ptx::mma_f16_ts_elect(tD, tA + k / 4u, ((uint64_t)hi << 32) | (lB + k / 16u), id, k > 0 ? 1u : 0u);
+        ptx::mma_commit_elect(bar);
+    }
+}
+
+// S (which = 0) or H (which = 1) of each slot once the value product of the slot
+// kRing before it has completed and the stage has landed (one probe: even lanes look
+// at one barrier, odd lanes at the other); an item's first slot also waits for the row
+// operands in TMEM.  One warp issuing both spent 600-800 cycles a slot on probes,
+// descriptors and instructions, against 380 of tensor work.  A bounded wait that runs
+// out makes the role go on without waits or tensor work, meeting its named barriers.
+__device__ void vjp_mma_sh(const VjpParams& p, VjpBarriers& bars, const uint8_t* sSt, const VjpSmem& m, uint32_t tmem,
+                           uint32_t which) {
+    const uint32_t row = (uint32_t)(which ? p.kh : p.k_pad) * 2u;
+    const uint32_t hi = ptx::smem_desc_hi(8u * row, swz_code(row));
+    const uint32_t id = ptx::idesc_f16(kBM, 64, 0);
+    const uint32_t lB0 = ptx::smem_desc_lo(ptx::smem_u32(sSt) + (which ? m.xbytes : 0u));
+    const uint32_t sh_full = ptx::smem_u32(&bars.sh_full[0]);
+    const uint32_t tA = tmem + (which ? kColUW : kColXA), tD = tmem + 64u * which;
+    const bool odd = threadIdx.x & 1;
+    uint32_t st = 0, ph = 0, b = 0, bph = 1;   // bph: parity of the buffer's last release (first round: passes at once)
     bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x, ++ic) {
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         int it, sp, j0, j1;
         item_range(p, item, it, sp, j0, j1);
-        const uint32_t T = (uint32_t)(j1 - j0);
-        const int xb = ic & 1;
-        if (!warp_wait(&bars.xi_full[xb], (ic >> 1) & 1, p.limit_ns)) { ok = false; break; }
-        ptx::tc_fence_after();
-        const uint32_t aXi = ptx::smem_u32(sXi) + (uint32_t)xb * m.xi_bytes;
-        for (uint32_t t = 0; t < T; ++t, ++g) {
-            if (g > 0 && !warp_wait(&bars.sh_empty, (g - 1) & 1, p.limit_ns)) { ok = false; break; }
-            if (!warp_wait(&bars.full[st], ph, p.limit_ns)) { ok = false; break; }
-            ptx::tc_fence_after();
-            const uint32_t aXj = aSt + st * m.stage_bytes;
-            for (int kk = 0; kk < p.k_pad / 16; ++kk)
-                ptx::mma_f16_ss_elect(tmem + kColS, ptx::smem_desc_at(hi_x, aXi + (uint32_t)kk * 32u),
-                                      ptx::smem_desc_at(hi_x, aXj + (uint32_t)kk * 32u), id, kk > 0 ? 1u : 0u);
-            for (int kk = 0; kk < p.kh / 16; ++kk)
-                ptx::mma_f16_ss_elect(tmem + kColH, ptx::smem_desc_at(hi_h, aXi + m.xbytes + (uint32_t)kk * 32u),
-                                      ptx::smem_desc_at(hi_h, aXj + m.xbytes + (uint32_t)kk * 32u), id,
-                                      kk > 0 ? 1u : 0u);
-            ptx::mma_commit_elect(&bars.sh_full);
-            if (t + 1 == T) ptx::mma_commit_elect(&bars.xi_empty[xb]);   // last use of the row tile
-            if (++st == S) { st = 0; ph ^= 1u; }
+        ptx::bar_sync(kBarA, kBarThreads + 32u);
+#pragma unroll 1
+        for (int jt = j0; jt < j1; ++jt) {
+            const uint32_t lB = lB0 + st * (m.stage_bytes >> 4);
+#pragma unroll 1
+            for (uint32_t h = 0; h < 2; ++h) {
+                ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(odd ? &bars.full[st] : &bars.w_empty[b],
+                                                                  odd ? ph : bph, p.limit_ns));
+                if (ok) {
+                    ptx::tc_fence_after();
+                    vjp_product(tD + b * 128u, tA, lB + h * 4u * row, row, hi, id, sh_full + 8u * b);
+                }
+                if (++b == kRing) { b = 0; bph ^= 1u; }
+            }
+            if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
         }
     }
-    ptx::mma_commit_elect(&bars.drain[0]);
-    warp_wait(&bars.drain[0], 0, p.limit_ns);
+    ptx::mma_commit_elect(&bars.drain[which]);
+    warp_wait(&bars.drain[which], 0, p.limit_ns);
     if (!ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
 }
 
 // ---- value-product issuer (one converged warp) ------------------------------------
-// O += W'(t) Xt_j^T with W' read from TMEM; then W' buffer t & 1 and the stage
-// are released.  O is handed to the epilogue at the end of an item.
+// O += W' Xt_j^T for each slot once its W' is stored; then the slot's buffer and,
+// after the tile's second slot, the stage are released.  O is handed to the
+// epilogue at the end of an item.
 __device__ void vjp_mma_o(const VjpParams& p, VjpBarriers& bars, const uint8_t* sSt, const VjpSmem& m,
                           uint32_t tmem) {
     const uint32_t hi_v = ptx::smem_desc_hi(1024u, 2u);
     const uint32_t id = ptx::idesc_f16(kBM, p.rv, 0);
-    const uint32_t S = (uint32_t)p.stages;
-    const uint32_t aSt = ptx::smem_u32(sSt);
-    const uint32_t vbox = (uint32_t)p.rv * 128u;
-    uint32_t g = 0, st = 0, ph = 0;
+    const uint32_t lV0 = ptx::smem_desc_lo(ptx::smem_u32(sSt) + m.xbytes + m.hbytes);
+    const uint32_t kb = (uint32_t)p.rv * 8u;   // a 64-column K-block in 16-byte units
+    const uint32_t w_empty = ptx::smem_u32(&bars.w_empty[0]);
+    uint32_t st = 0, ph = 0, b = 0;
     int ic = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x, ++ic) {
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int it, sp, j0, j1;
         item_range(p, item, it, sp, j0, j1);
-        const uint32_t T = (uint32_t)(j1 - j0);
-        for (uint32_t t = 0; t < T; ++t, ++g) {
-            if (t == 0 && ic > 0 && !warp_wait(&bars.o_empty, (ic - 1) & 1, p.limit_ns)) { ok = false; break; }
-            if (!warp_wait(&bars.full[st], ph, p.limit_ns)) { ok = false; break; }   // Xt_j: landed for S
-            const uint32_t wb = g & 1u;
-            if (!warp_wait(&bars.w_full[wb], (g >> 1) & 1, p.limit_ns)) { ok = false; break; }
-            ptx::tc_fence_after();
-            const uint32_t aV = aSt + st * m.stage_bytes + m.xbytes + m.hbytes;
-#pragma unroll
-            for (int kk = 0; kk < kBN / 16; ++kk) {
-                const uint32_t off = (uint32_t)(kk >> 2) * vbox + (uint32_t)(kk & 3) * 32u;
-                ptx::mma_f16_ts_elect(tmem + kColO, tmem + kColW + wb * 64u + (uint32_t)kk * 8u,
-                                      ptx::smem_desc_at(hi_v, aV + off), id, (t > 0 || kk > 0) ? 1u : 0u);
+        if (ic > 0) ok = ok && warp_wait(&bars.o_empty, (ic - 1) & 1, p.limit_ns);
+#pragma unroll 1
+        for (int jt = j0; jt < j1; ++jt) {
+            ok = ok && warp_wait(&bars.full[st], ph, p.limit_ns);   // Xt_j: landed for S
+            const uint32_t lV = lV0 + st * (m.stage_bytes >> 4);
+#pragma unroll 1
+            for (uint32_t h = 0; h < 2; ++h) {
+                ptx::bar_sync(kBarW + b, kBarThreads);
+                if (ok) {
+                    ptx::tc_fence_after();
+                    ptx::mma_f16_ts4_elect<8, 32, 40>(tmem + kColO, tmem + b * 128u, lV + h * kb, hi_v, id,
+                                                      (jt > j0 || h > 0) ? 1u : 0u, w_empty + 8u * b);
+                }
+                if (++b == kRing) b = 0;
             }
-            ptx::mma_commit_elect(&bars.w_empty[wb]);   // W' buffer wb may be rewritten
-            ptx::mma_commit_elect(&bars.empty[st]);     // the stage's operands are consumed
-            if (++st == S) { st = 0; ph ^= 1u; }
+            if (ok) ptx::mma_commit_elect(&bars.empty[st]);     // the stage's operands are consumed
+            if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
         }
-        if (!ok) break;
-        ptx::mma_commit_elect(&bars.o_full);
+        if (ok) ptx::mma_commit_elect(&bars.o_full);
     }
-    ptx::mma_commit_elect(&bars.drain[1]);
-    warp_wait(&bars.drain[1], 0, p.limit_ns);
+    ptx::mma_commit_elect(&bars.drain[2]);
+    warp_wait(&bars.drain[2], 0, p.limit_ns);
     if (!ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
 }
 
@@ -265,30 +299,62 @@ __device__ __forceinline__ void wprime(float s, float h, float& w, float& hk) {
     }
 }
 
+// A row operand of an item from its swizzled shared-memory tile (rows of `row`
+// bytes) into TMEM: this thread's row, 16-byte chunks in K order, 4 columns each.
+__device__ __forceinline__ void vjp_row_to_tmem(uint32_t sT, uint32_t row, uint32_t r, uint32_t tA) {
+    const uint32_t mask = row / 16u - 1u;   // chunks per row - 1 = the swizzle's address bits
+    for (uint32_t c = 0; c < row / 16u; c += 2) {
+        uint32_t v[8];
+#pragma unroll
+        for (uint32_t u = 0; u < 2; ++u) {
+            const uint32_t off = r * row + (c + u) * 16u;
+            const uint32_t phys = off ^ (((off >> 7) & mask) << 4);
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v[4 * u]), "=r"(v[4 * u + 1]), "=r"(v[4 * u + 2]), "=r"(v[4 * u + 3])
+                         : "r"(sT + phys));
+        }
+        ptx::tmem_st8(tA + c * 4u, v);
+    }
+}
+
 template <int KIND>
-__device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, uint32_t tmem, int q, int wq, int lane,
-                             double* red) {
+__device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, const uint8_t* sXi, const VjpSmem& m, uint32_t tmem,
+                             int wg, int wq, int lane, double* red) {
+    const int pr = wg & 1, ch = wg >> 1;              // slot parity (half of a tile), half of its 64 columns
     const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
-    uint32_t g = 0;
+    uint32_t b = (uint32_t)pr, ph = 0;                // ring slot of this warp's next slot and its fill parity
     int ic = 0;
     bool ok = true;
     double acc = 0.0;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x, ++ic) {
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int it, sp, j0, j1;
         item_range(p, item, it, sp, j0, j1);
-        const uint32_t T = (uint32_t)(j1 - j0);
-        for (uint32_t t = 0; t < T; ++t, ++g) {
-            if (!warp_wait(&bars.sh_full, g & 1, p.limit_ns)) { ok = false; break; }
+        if (pr == 0) {
+            // warpgroup 0: XA_i, warpgroup 2: UW_i.  The products of the last item that read them are done
+            // (its O was complete).
+            ok = ok && warp_wait(&bars.xi_full[ic & 1], (ic >> 1) & 1, p.limit_ns);
+            const uint32_t sX = ptx::smem_u32(sXi) + (uint32_t)(ic & 1) * m.xi_bytes;
+            const uint32_t r = (uint32_t)(wq * 32 + lane);
+            if (ch == 0) vjp_row_to_tmem(sX, (uint32_t)p.k_pad * 2u, r, tmem + lane_off + kColXA);
+            else vjp_row_to_tmem(sX + m.xbytes, (uint32_t)p.kh * 2u, r, tmem + lane_off + kColUW);
+            ptx::tmem_wait_st();
+            ptx::tc_fence_before();
+            ptx::bar_arrive(kBarA, kBarThreads + 32u, ok);
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&bars.xi_empty[ic & 1]);
+        }
+#pragma unroll 1
+        for (int jt = j0; jt < j1; ++jt) {
+            ok = ok && warp_wait(&bars.sh_full[b], ph, p.limit_ns);
             ptx::tc_fence_after();
+            const uint32_t tS = tmem + lane_off + b * 128u + (uint32_t)ch * 32u;
             uint32_t rs[32], rh[32];
-            ptx::tmem_ld32(tmem + lane_off + kColS + (uint32_t)q * 32u, rs);
-            ptx::tmem_ld32(tmem + lane_off + kColH + (uint32_t)q * 32u, rh);
+            ptx::tmem_ld32(tS, rs);
+            ptx::tmem_ld32(tS + 64u, rh);
             ptx::tmem_wait_ld();
             ptx::tmem_reg_fence(rs);
             ptx::tmem_reg_fence(rh);
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars.sh_empty);   // this warp's part of S and H is in registers
             uint32_t pk[16];
             float a = 0.0f;
 #pragma unroll
@@ -300,30 +366,21 @@ __device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, uint32_t tme
                 __half2 hv = __floats2half2_rn(w0, w1);
                 pk[e] = *reinterpret_cast<uint32_t*>(&hv);
             }
-            acc += (double)a;
-            const uint32_t wb = g & 1u;
-            if (g >= 2 && !warp_wait(&bars.w_empty[wb], ((g >> 1) - 1) & 1, p.limit_ns)) { ok = false; break; }
-            ptx::tmem_st16(tmem + lane_off + kColW + wb * 64u + (uint32_t)q * 16u, pk);
+            ptx::tmem_st16(tS, pk);
             ptx::tmem_wait_st();
             ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars.w_full[wb]);
+            ptx::bar_arrive(kBarW + b, kBarThreads, ok);
+            acc += (double)a;   // FP64 is slow here: behind the arrival
+            b += 2;
+            if (b >= kRing) { b -= kRing; ph ^= 1u; }
         }
-        if (!ok) break;
-        // O read-out: this warpgroup's rv / 4 columns of its 32 rows
-        if (!warp_wait(&bars.o_full, ic & 1, p.limit_ns)) { ok = false; break; }
+        // O read-out in chunks of 8 columns, dealt to the warpgroups
+        ok = ok && warp_wait(&bars.o_full, ic & 1, p.limit_ns);
         ptx::tc_fence_after();
         const int64_t row = (int64_t)it * kBM + wq * 32 + lane;
-        const int ncol = p.rv / 4, c0 = q * ncol;
-        float* dst = p.part + ((int64_t)sp * p.rv + c0) * p.N_pad + row;
-        if (ncol == 16) {
-            uint32_t o[16];
-            ptx::tmem_ld16(tmem + lane_off + kColO + (uint32_t)c0, o);
-            ptx::tmem_wait_ld();
-            ptx::tmem_reg_fence(o);
-#pragma unroll
-            for (int c = 0; c < 16; ++c) dst[(int64_t)c * p.N_pad] = __uint_as_float(o[c]);
-        } else {
+#pragma unroll 1
+        for (int c0 = 8 * wg; c0 < p.rv; c0 += 32) {
+            float* dst = p.part + ((int64_t)sp * p.rv + c0) * p.N_pad + row;
             uint32_t o[8];
             ptx::tmem_ld8(tmem + lane_off + kColO + (uint32_t)c0, o);
             ptx::tmem_wait_ld();
@@ -338,7 +395,7 @@ __device__ void vjp_epilogue(const VjpParams& p, VjpBarriers& bars, uint32_t tme
     if (!ok && lane == 0) record_error(p.err, DEV_TIMEOUT);
     // per-CTA sum of H k in a fixed order: warp shuffle tree, then the warps in order
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) red[q * 4 + wq] = acc;
+    if (lane == 0) red[wg * 4 + wq] = acc;
 }
 
 template <int KIND>
@@ -351,24 +408,25 @@ kvjp_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __shared__ uint32_t tmem_slot;
     __shared__ double red[kEpiWarps];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~uintptr_t(1023));
-    const VjpSmem m = vjp_smem(p.k_pad, p.kh, p.rv);
+    const VjpSmem& m = p.sm;
     uint8_t* sSt = base;
     uint8_t* sXi = base + (uint32_t)p.stages * m.stage_bytes;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform
     if (threadIdx.x == 0) {
+#pragma unroll 1
         for (int s = 0; s < kMaxStages; ++s) {
             ptx::mbar_init(&bars.full[s], 1);
             ptx::mbar_init(&bars.empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&bars.xi_full[b], 1);
-            ptx::mbar_init(&bars.xi_empty[b], 1);
-            ptx::mbar_init(&bars.w_full[b], kEpiWarps);   // one arrival per epilogue warp
-            ptx::mbar_init(&bars.w_empty[b], 1);
-            ptx::mbar_init(&bars.drain[b], 1);
+            ptx::mbar_init(&bars.xi_empty[b], 8);         // the warps that copy the row operands
         }
-        ptx::mbar_init(&bars.sh_full, 1);
-        ptx::mbar_init(&bars.sh_empty, kEpiWarps);
+        for (uint32_t b = 0; b < 3; ++b) ptx::mbar_init(&bars.drain[b], 1);
+        for (uint32_t b = 0; b < kRing; ++b) {
+            ptx::mbar_init(&bars.sh_full[b], 2);          // the S and the H issuer
+            ptx::mbar_init(&bars.w_empty[b], 1);
+        }
         ptx::mbar_init(&bars.o_full, 1);
         ptx::mbar_init(&bars.o_empty, kEpiWarps);
         ptx::fence_mbar_init();
@@ -388,12 +446,12 @@ kvjp_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (warp == kTmaWarp) {
         if (lane == 0) vjp_producer(p, &tmA, &tmB, &tmUW, &tmWU, &tmXt, bars, sSt, sXi, m);
         __syncwarp();
-    } else if (warp == kShWarp) {
-        vjp_mma_sh(p, bars, sSt, sXi, m, tmem);
+    } else if (warp == kShWarp || warp == kShWarp + 1) {
+        vjp_mma_sh(p, bars, sSt, m, tmem, (uint32_t)(warp - kShWarp));
     } else if (warp == kOWarp) {
         vjp_mma_o(p, bars, sSt, m, tmem);
     } else {
-        vjp_epilogue<KIND>(p, bars, tmem, warp >> 2, warp & 3, lane, red);
+        vjp_epilogue<KIND>(p, bars, sXi, m, tmem, warp >> 2, warp & 3, lane, red);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -488,7 +546,7 @@ __global__ void __launch_bounds__(256)
 vjp_finish_kernel(const float* __restrict__ part, int n_split, int rv, int64_t N_pad, const float* __restrict__ xs,
                   const float* __restrict__ Vb, int64_t N, int d, ScaleVec two_over_l, float a2kp,
                   const float* __restrict__ scales, int rp, float* __restrict__ gX, double* __restrict__ lpart) {
-    const int rx = rv / 2;
+    const int rx = d + 1;
     const float g = scales[rp];
     const float F = a2kp / (g * g);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -604,8 +662,8 @@ VjpPlan vjp_plan(const Ctx* ctx, const KOp& op, int64_t N, int d, int R) {
     p.n_jt = (int)(p.Nc_pad / kBN);
     p.rp = R <= 16 ? 16 : 32;
     p.kh = 2 * p.rp;
-    p.rx = (d + 1) <= 16 ? 16 : 32;
-    p.rv = 2 * p.rx;
+    p.rx = d + 1;                                  // rows of Xt per part: hi, then lo
+    p.rv = ((2 * p.rx + 15) / 16) * 16;
     const int G = ctx->num_sms > 0 ? ctx->num_sms : 1;
     // column split minimising the busiest CTA's tiles (+ about two tiles of per-item cost)
     int best = 1;
@@ -696,7 +754,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     ctx->launches += 3;
     if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
     GPK_TRY(launch_v_colmax(ctx, Vb, N, d + 1, cmv, s));
-    GPK_TRY(launch_v_cast(ctx, GP_PREC_FP16, 0, 1, Vb, N, pl.Nc_pad, d + 1, pl.rx, 2 * pl.rx, cmv, 1.0, Xt, xs, s));
+    GPK_TRY(launch_v_cast(ctx, GP_PREC_FP16, 0, 1, Vb, N, pl.Nc_pad, d + 1, pl.rx, pl.rv, cmv, 1.0, Xt, xs, s));
 
     CUtensorMap tmUW, tmWU, tmXt;
     const uint32_t hrow = (uint32_t)pl.kh * 2u;
@@ -718,6 +776,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
     const VjpSmem m = vjp_smem(prm.k_pad, prm.kh, prm.rv);
     if (m.stages < 2) return GP_ERR_UNSUPPORTED;
     prm.stages = m.stages;
+    prm.sm = m;
     prm.N_pad = pl.N_pad;
     prm.part = part;
     prm.hk = hk;

@@ -525,8 +525,12 @@ def test_pair_engine_tile_edges(ctx, mode, N, R):
 def test_fp32_few_rows_many_splits(ctx, Nr, R):
     """The FP32 engine on few rows and many columns (the posterior mean): more
     than 64 column splits with 1 to 3 vectors, and their reduction, at the edges
-    of its 32-row blocks and of the column tiles."""
+    of its 32-row blocks and of the column tiles.  Each output against the FP32
+    tolerance times the sum of its terms' magnitudes: a single output of
+    random-sign vectors cancels, so it has no small error relative to itself."""
     X, V, _, ls, a2, s2 = workloads.random_problem(20_001, 7, R, seed=Nr + R, kernel=1)
     Xr = np.random.default_rng(Nr).standard_normal((Nr, 7)).astype(np.float32)
     got = _run(ctx, Xr, V, 1, ls, a2, s2, "fp32", Xc=X, add_noise=False)
-    assert _colerr(got, _ref(Xr, V, 1, ls, a2, s2, Xc=X, add_noise=False)) <= TOL["fp32"]
+    ref = _ref(Xr, V, 1, ls, a2, s2, Xc=X, add_noise=False)
+    mag = _ref(Xr, np.abs(V), 1, ls, a2, s2, Xc=X, add_noise=False)
+    assert np.all(np.abs(got - ref) <= TOL["fp32"] * mag)
