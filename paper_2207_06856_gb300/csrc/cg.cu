@@ -103,6 +103,35 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float bh, float bl)
     lo = __fadd_rn(__fadd_rn(lo, bl), e);
 }
 
+// Block sums of a 2048-element chunk from each thread's float-float sums of a b
+// (sh, sl) and a^2 (nh, nl): through the warp and the 8 warps of a 256-thread group
+// in a fixed order; `sw` holds the group's 8 warp sums.  Thread 0 of the group
+// writes (s, e, sum a^2) to o.  sync(): a barrier of the group.
+template <class Sync>
+__device__ __forceinline__ void dots_reduce(float sh, float sl, float nh, float nl, int t, float4* sw, double* o,
+                                            Sync sync) {
+    for (int off = 16; off > 0; off >>= 1) {
+        const float h1 = __shfl_xor_sync(0xffffffffu, sh, off), l1 = __shfl_xor_sync(0xffffffffu, sl, off);
+        const float h2 = __shfl_xor_sync(0xffffffffu, nh, off), l2 = __shfl_xor_sync(0xffffffffu, nl, off);
+        ff_add(sh, sl, h1, l1);
+        ff_add(nh, nl, h2, l2);
+    }
+    if ((t & 31) == 0) sw[t >> 5] = make_float4(sh, sl, nh, nl);
+    sync();
+    if (t == 0) {
+        float4 u = sw[0];
+        for (int q = 1; q < kDotThreads / 32; ++q) {
+            ff_add(u.x, u.y, sw[q].x, sw[q].y);
+            ff_add(u.z, u.w, sw[q].z, sw[q].w);
+        }
+        Lse acc{0.0, kEmptyExp};
+        lse_add(acc, (double)u.x + (double)u.y);
+        o[0] = acc.s;
+        o[1] = (double)acc.e;
+        o[2] = (double)u.z + (double)u.w;
+    }
+}
+
 // part[(c * nblk + blk) * 3 + {0,1,2}] = (s, e, sum a^2) of column c over this chunk.
 __global__ void __launch_bounds__(kDotThreads)
 dots_kernel(const float* __restrict__ A, const float* __restrict__ B, int64_t N, int nblk,
@@ -127,147 +156,137 @@ dots_kernel(const float* __restrict__ A, const float* __restrict__ B, int64_t N,
             ff_add_prod(nh, nl, av, av);
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h1 = __shfl_xor_sync(0xffffffffu, sh, o), l1 = __shfl_xor_sync(0xffffffffu, sl, o);
-        const float h2 = __shfl_xor_sync(0xffffffffu, nh, o), l2 = __shfl_xor_sync(0xffffffffu, nl, o);
-        ff_add(sh, sl, h1, l1);
-        ff_add(nh, nl, h2, l2);
-    }
     __shared__ float4 sw[kDotThreads / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sw[w] = make_float4(sh, sl, nh, nl);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float4 t = sw[0];
-        for (int q = 1; q < kDotThreads / 32; ++q) {
-            ff_add(t.x, t.y, sw[q].x, sw[q].y);
-            ff_add(t.z, t.w, sw[q].z, sw[q].w);
-        }
-        Lse acc{0.0, kEmptyExp};
-        lse_add(acc, (double)t.x + (double)t.y);
-        double* o = part + ((int64_t)c * nblk + blockIdx.x) * 3;
-        o[0] = acc.s;
-        o[1] = (double)acc.e;
-        o[2] = (double)t.z + (double)t.w;
-    }
+    dots_reduce(sh, sl, nh, nl, (int)threadIdx.x, sw, part + ((int64_t)c * nblk + blockIdx.x) * 3,
+                [] { __syncthreads(); });
 }
 
 enum ScalarMode { SC_INIT = 0, SC_ALPHA = 1, SC_BETA = 2, SC_BNORM = 3 };
 
+// The scalar step of column c by one warp (lane l): merge the column's partials
+// (part: its nblk triples) in a fixed order, then the step of Alg. 1 / Alg. 2.
+__device__ void scalar_column(int mode, int stable, const double* part, int nblk, int R, ColState* __restrict__ st, int c,
+                              int l, int k, double tol, int min_iter, double* __restrict__ ahist,
+                              double* __restrict__ bhist, double* __restrict__ rhist, int* __restrict__ n_active,
+                              int* __restrict__ aflags) {
+    ColState& S = st[c];
+    const bool act = (mode == SC_INIT || mode == SC_BNORM) ? true : (S.active != 0);
+    if (act) {
+        Lse acc{0.0, kEmptyExp};
+        double n2 = 0.0;
+        for (int b = l; b < nblk; b += 32) {
+            const double* o = part + (int64_t)b * 3;
+            lse_merge(acc, Lse{o[0], (int)o[1]});
+            n2 += o[2];
+        }
+        // fixed-order tree merge across lanes
+        for (int off = 16; off > 0; off >>= 1) {
+            lse_merge(acc, lse_shfl(acc, off));
+            n2 += __shfl_xor_sync(0xffffffffu, n2, off);
+        }
+        if (l == 0) {
+            // acc = (s, e) with LSE = log s + e log 2; Alg. 2's
+            // exp(LSE_1 - LSE_2) is formed as ldexp(s_1 / s_2, e_1 - e_2):
+            // the same quotient, no transcendental, no overflow.
+            const bool pos = acc.e != kEmptyExp && acc.s > 0.0;
+            const double val = pos ? ldexp(acc.s, acc.e) : 0.0;
+            if (mode == SC_BNORM) {
+                S.bnorm = sqrt(n2);
+            } else if (mode == SC_INIT) {
+                S.rnorm = sqrt(n2);
+                S.relres = S.bnorm > 0.0 ? S.rnorm / S.bnorm : 0.0;
+                S.gamma_s = pos ? acc.s : 0.0;
+                S.gamma_e = pos ? acc.e : 0;
+                S.gamma = val;
+                // r_0^T z_0 of the first run only: it weights the SLQ quadrature
+                // of the Lanczos process that run's step sizes describe, and a
+                // true-residual restart (k > 0) must not overwrite it
+                if (k == 0) S.gamma0 = val;
+                S.alpha = 0.0;
+                S.beta = 0.0;
+                S.iters = k;
+                S.breakdown = 0;
+                const bool work = S.bnorm > 0.0 && S.rnorm > 0.0 && (S.relres > tol || min_iter > k);
+                if (work && !pos) S.breakdown = 1;
+                S.active = (work && pos) ? 1 : 0;
+                if (rhist) rhist[(int64_t)k * R + c] = S.relres;
+            } else if (mode == SC_ALPHA) {
+                // alpha_k = gamma_k / d^T K d  (Alg. 2: from the LSE forms)
+                if (!pos) {
+                    S.breakdown = 1;
+                    S.active = 0;
+                    S.alpha = 0.0;
+                } else {
+                    S.alpha = stable ? ldexp(S.gamma_s / acc.s, S.gamma_e - acc.e) : S.gamma / val;
+                }
+                if (ahist) ahist[(int64_t)k * R + c] = S.alpha;
+            } else {   // SC_BETA
+                S.rnorm = sqrt(n2);
+                S.relres = S.bnorm > 0.0 ? S.rnorm / S.bnorm : 0.0;
+                S.iters = k + 1;
+                if (rhist) rhist[(int64_t)(k + 1) * R + c] = S.relres;
+                if (S.rnorm == 0.0) {
+                    S.active = 0;           // exact solution reached
+                    S.beta = 0.0;
+                } else if (!pos) {
+                    S.breakdown = 1;
+                    S.active = 0;
+                    S.beta = 0.0;
+                } else {
+                    S.beta = stable ? ldexp(acc.s / S.gamma_s, acc.e - S.gamma_e) : val / S.gamma;
+                    S.gamma_s = acc.s;
+                    S.gamma_e = acc.e;
+                    S.gamma = val;
+                    if (bhist) bhist[(int64_t)k * R + c] = S.beta;
+                    if (S.relres <= tol && k + 1 >= min_iter) S.active = 0;
+                }
+            }
+            if (S.breakdown && n_active) atomicAdd(&n_active[1], 1);   // breakdowns of this run
+        }
+    }
+    if (l == 0 && aflags) aflags[c] = S.active;   // the masks of the masked kernels
+}
+
+// The last block of the grid to come here counts the active columns (n_active[2] is
+// its ticket, returned to 0 by that block).  One warp per block.
+__device__ void scalar_ticket(const ColState* __restrict__ st, int R, int l, int* __restrict__ n_active) {
+    int last = 0;
+    if (l == 0) {
+        __threadfence();
+        last = atomicAdd(&n_active[2], 1) == (int)gridDim.x - 1;
+    }
+    if (__shfl_sync(0xffffffffu, last, 0)) {
+        __threadfence();
+        int cnt = 0;
+        float rmax = 0.0f;   // largest recursive relative residual of the active columns
+        for (int q = l; q < R; q += 32) {
+            if (*(volatile const int*)&st[q].active != 0) {
+                ++cnt;
+                rmax = fmaxf(rmax, (float)*(volatile const double*)&st[q].relres);
+            }
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        const unsigned rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));   // non-negative floats
+        if (l == 0) {
+            n_active[0] = cnt;
+            n_active[2] = 0;
+            n_active[3] = (int)rbits;
+        }
+    }
+}
+
 // One block of one warp per column, so the FP64 merges and recurrences of the
 // columns run on different SMs (FP64 throughput is per SM and low on this
 // GPU): merge the partials of column c in a fixed order, then run the scalar
-// step of Alg. 1 / Alg. 2.  The last block to finish counts the active
-// columns (n_active[2] is its ticket, returned to 0 by that block).
+// step of Alg. 1 / Alg. 2.
 __global__ void __launch_bounds__(32)
 scalar_kernel(int mode, int stable, const double* __restrict__ part, int nblk, int R, ColState* __restrict__ st,
               int k, double tol, int min_iter, double* __restrict__ ahist, double* __restrict__ bhist,
               double* __restrict__ rhist, int* __restrict__ n_active, int* __restrict__ aflags) {
-    const int l = threadIdx.x;
-    {
-        const int c = blockIdx.x;
-        ColState& S = st[c];
-        const bool act = (mode == SC_INIT || mode == SC_BNORM) ? true : (S.active != 0);
-        if (act) {
-            Lse acc{0.0, kEmptyExp};
-            double n2 = 0.0;
-            for (int b = l; b < nblk; b += 32) {
-                const double* o = part + ((int64_t)c * nblk + b) * 3;
-                lse_merge(acc, Lse{o[0], (int)o[1]});
-                n2 += o[2];
-            }
-            // fixed-order tree merge across lanes
-            for (int off = 16; off > 0; off >>= 1) {
-                lse_merge(acc, lse_shfl(acc, off));
-                n2 += __shfl_xor_sync(0xffffffffu, n2, off);
-            }
-            if (l == 0) {
-                // acc = (s, e) with LSE = log s + e log 2; Alg. 2's
-                // exp(LSE_1 - LSE_2) is formed as ldexp(s_1 / s_2, e_1 - e_2):
-                // the same quotient, no transcendental, no overflow.
-                const bool pos = acc.e != kEmptyExp && acc.s > 0.0;
-                const double val = pos ? ldexp(acc.s, acc.e) : 0.0;
-                if (mode == SC_BNORM) {
-                    S.bnorm = sqrt(n2);
-                } else if (mode == SC_INIT) {
-                    S.rnorm = sqrt(n2);
-                    S.relres = S.bnorm > 0.0 ? S.rnorm / S.bnorm : 0.0;
-                    S.gamma_s = pos ? acc.s : 0.0;
-                    S.gamma_e = pos ? acc.e : 0;
-                    S.gamma = val;
-                    // r_0^T z_0 of the first run only: it weights the SLQ quadrature
-                    // of the Lanczos process that run's step sizes describe, and a
-                    // true-residual restart (k > 0) must not overwrite it
-                    if (k == 0) S.gamma0 = val;
-                    S.alpha = 0.0;
-                    S.beta = 0.0;
-                    S.iters = k;
-                    S.breakdown = 0;
-                    const bool work = S.bnorm > 0.0 && S.rnorm > 0.0 && (S.relres > tol || min_iter > k);
-                    if (work && !pos) S.breakdown = 1;
-                    S.active = (work && pos) ? 1 : 0;
-                    if (rhist) rhist[(int64_t)k * R + c] = S.relres;
-                } else if (mode == SC_ALPHA) {
-                    // alpha_k = gamma_k / d^T K d  (Alg. 2: from the LSE forms)
-                    if (!pos) {
-                        S.breakdown = 1;
-                        S.active = 0;
-                        S.alpha = 0.0;
-                    } else {
-                        S.alpha = stable ? ldexp(S.gamma_s / acc.s, S.gamma_e - acc.e) : S.gamma / val;
-                    }
-                    if (ahist) ahist[(int64_t)k * R + c] = S.alpha;
-                } else {   // SC_BETA
-                    S.rnorm = sqrt(n2);
-                    S.relres = S.bnorm > 0.0 ? S.rnorm / S.bnorm : 0.0;
-                    S.iters = k + 1;
-                    if (rhist) rhist[(int64_t)(k + 1) * R + c] = S.relres;
-                    if (S.rnorm == 0.0) {
-                        S.active = 0;           // exact solution reached
-                        S.beta = 0.0;
-                    } else if (!pos) {
-                        S.breakdown = 1;
-                        S.active = 0;
-                        S.beta = 0.0;
-                    } else {
-                        S.beta = stable ? ldexp(acc.s / S.gamma_s, acc.e - S.gamma_e) : val / S.gamma;
-                        S.gamma_s = acc.s;
-                        S.gamma_e = acc.e;
-                        S.gamma = val;
-                        if (bhist) bhist[(int64_t)k * R + c] = S.beta;
-                        if (S.relres <= tol && k + 1 >= min_iter) S.active = 0;
-                    }
-                }
-                if (S.breakdown && n_active) atomicAdd(&n_active[1], 1);   // breakdowns of this run
-            }
-        }
-        if (l == 0 && aflags) aflags[c] = S.active;   // the masks of the masked kernels
-    }
-    if (n_active) {
-        int last = 0;
-        if (l == 0) {
-            __threadfence();
-            last = atomicAdd(&n_active[2], 1) == (int)gridDim.x - 1;
-        }
-        if (__shfl_sync(0xffffffffu, last, 0)) {
-            __threadfence();
-            int cnt = 0;
-            float rmax = 0.0f;   // largest recursive relative residual of the active columns
-            for (int q = l; q < R; q += 32) {
-                if (*(volatile const int*)&st[q].active != 0) {
-                    ++cnt;
-                    rmax = fmaxf(rmax, (float)*(volatile const double*)&st[q].relres);
-                }
-            }
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            const unsigned rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));   // non-negative floats
-            if (l == 0) {
-                n_active[0] = cnt;
-                n_active[2] = 0;
-                n_active[3] = (int)rbits;
-            }
-        }
-    }
+    const int c = blockIdx.x;
+    scalar_column(mode, stable, part + (int64_t)c * nblk * 3, nblk, R, st, c, threadIdx.x, k, tol, min_iter, ahist, bhist,
+                  rhist, n_active, aflags);
+    if (n_active) scalar_ticket(st, R, threadIdx.x, n_active);
 }
 
 // x += alpha d; r += alpha Kd   (active columns)
@@ -426,6 +445,297 @@ __global__ void reorth_update_kernel(const float* __restrict__ RB, int nb, int R
 
 
 
+// ---- the rest of an iteration of a small system in one launch ---------------------
+// Everything between two MVMs is per column: one CTA per column runs it with block
+// barriers where the kernels above need a launch each (13 launches of 2-8 us for a
+// few thousand rows; one request of N = 2,000, rank 20, spent 115 us an iteration,
+// 7 of them in its MVM).  Thread t of group g (256 threads) owns elements
+// 2048 g + 256 q + t, q < 8, as in dots_kernel's chunks, with r and z in registers.
+// Every sum runs in the order of the kernels it stands for, so the results are the
+// same bit for bit: the split sums of the MVM, the float-float dots, the Gram
+// coefficients, the Woodbury apply (32-row blocks, FP64 across them).
+constexpr int kTailMaxN = 4 * kDotChunk;
+constexpr int kTailThreads = 1024;
+struct TailParams {
+    int N, R, nblk, k, nb, passes, reorth, stable, rank, min_iter;
+    double tol;
+    float *x, *r, *d;
+    const float* Kd;        // the MVM's result, or null: its partial sums
+    MvmParts mv;
+    const float* ZB;        // basis the Gram coefficients are taken with
+    const float* RB;        // basis the projection subtracts
+    float *rho_k, *zeta_k;  // this iterate's basis vectors
+    const float* L;
+    const double* cinv;
+    float inv_s2, inv_s4;
+    ColState* st;
+    double *ahist, *bhist, *rhist;
+    int *nact, *aflags;
+    float* v32;             // FP32 copy of d for the next MVM (row stride ld_v32), or null
+    float* outscale;
+    int64_t ld_v32;
+    float a2;
+    int* err;
+};
+
+size_t tail_smem(int N) {
+    // part 16, gram sums 128, t 512 doubles; warp sums 32 float4; Gram 1024, coefficients 1024, u 512 floats;
+    // r with one word of padding per 32; a 32 x 33 staging tile per warp
+    return (16 + 128 + 512) * sizeof(double) + 32 * sizeof(float4) +
+           (1024 + 1024 + 512 + (size_t)(N + N / 32 + 33) + 32 * 32 * 33) * sizeof(float);
+}
+
+__global__ void __launch_bounds__(kTailThreads, 1) cg_tail_kernel(const TailParams p) {
+    extern __shared__ double tsm[];
+    double* part = tsm;
+    double* gp = part + 16;                                 // [4][32]
+    double* tv = gp + 128;                                  // t = L^T r
+    float4* sw = reinterpret_cast<float4*>(tv + 512);       // [4][8]
+    float* sred = reinterpret_cast<float*>(sw + 32);        // [4][8][32]
+    float* sc = sred + 1024;                                // projection coefficients
+    float* su = sc + 1024;                                  // u = C^{-1} t
+    float* tile = su + 512;                                 // [32 warps][32][33]
+    float* sr = tile + 32 * 32 * 33;                        // r, index i + i / 32
+    __shared__ float s_beta, s_sg;
+    const int c = blockIdx.x, tid = threadIdx.x, g = tid >> 8, t = tid & 255, w = tid >> 5, l = tid & 31;
+    const int N = p.N;
+    const int64_t col = (int64_t)c * N;
+    const int i0 = g * kDotChunk + t;                       // element q: i0 + 256 q
+    ColState& S = p.st[c];
+    volatile const int* active = &S.active;
+    volatile const double* alpha = &S.alpha;
+    const auto sync = [] { __syncthreads(); };
+
+    if (*active) {
+        // Kd (from the MVM's split sums where it left them), d^T K d and alpha
+        float kd[kDotPerThread], rv[kDotPerThread];
+        float sh = 0.0f, sl = 0.0f, nh = 0.0f, nl = 0.0f;
+        const float osc = p.Kd ? 0.0f : p.mv.outscale[c];
+#pragma unroll
+        for (int q = 0; q < kDotPerThread; ++q) {
+            const int i = i0 + q * kDotThreads;
+            kd[q] = 0.0f;
+            if (i < N) {
+                const float dv = p.d[col + i];
+                if (p.Kd) {
+                    kd[q] = p.Kd[col + i];
+                } else {
+                    float sum = 0.0f;
+#pragma unroll 8
+                    for (int u = 0; u < p.mv.parts; ++u) sum += p.mv.partial[((int64_t)u * p.R + c) * p.mv.ld + i];
+                    float v = sum * osc;
+                    if (p.mv.noise != 0.0f) v = fmaf(p.mv.noise, dv, v);
+                    kd[q] = v;
+                }
+                ff_add_prod(sh, sl, dv, kd[q]);
+                ff_add_prod(nh, nl, dv, dv);
+            }
+        }
+        dots_reduce(sh, sl, nh, nl, t, sw + 8 * g, part + 3 * g, sync);
+        __syncthreads();
+        if (w == 0)
+            scalar_column(SC_ALPHA, p.stable, part, p.nblk, p.R, p.st, c, l, p.k, p.tol, p.min_iter, p.ahist, p.bhist,
+                          p.rhist, p.nact, p.aflags);
+        __syncthreads();
+        if (*active) {
+            const float a = (float)*alpha;
+#pragma unroll
+            for (int q = 0; q < kDotPerThread; ++q) {
+                const int i = i0 + q * kDotThreads;
+                rv[q] = 0.0f;
+                if (i < N) {
+                    p.x[col + i] = fmaf(a, p.d[col + i], p.x[col + i]);
+                    rv[q] = fmaf(a, kd[q], p.r[col + i]);
+                }
+            }
+            // re-orthogonalisation: all coefficients, then the projection, per pass
+            const int64_t stride = (int64_t)p.R * N;
+            if (p.reorth != GP_REORTH_NONE) {
+                for (int pass = 0; pass < p.passes; ++pass) {
+                    for (int jb = 0; jb < p.nb; jb += 32) {
+                        const int cnt = p.nb - jb < 32 ? p.nb - jb : 32;
+                        const float* zb = p.ZB + (int64_t)jb * stride + col;
+                        for (int j = 0; j < cnt; j += 4) {
+                            float av[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                            for (int q = 0; q < kDotPerThread; ++q) {
+                                const int i = i0 + q * kDotThreads;
+                                if (i < N) {
+#pragma unroll
+                                    for (int u = 0; u < 4; ++u)
+                                        if (j + u < cnt) av[u] = fmaf(zb[(int64_t)(j + u) * stride + i], rv[q], av[u]);
+                                }
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                for (int o = 16; o > 0; o >>= 1) av[u] += __shfl_xor_sync(0xffffffffu, av[u], o);
+                                if (l == 0 && j + u < cnt) sred[w * 32 + j + u] = av[u];
+                            }
+                        }
+                        __syncthreads();
+                        if (w < p.nblk && l < cnt) {   // warp w: chunk w's 8 warp sums
+                            double v = 0.0;
+                            for (int q = 0; q < 8; ++q) v += (double)sred[(8 * w + q) * 32 + l];
+                            gp[w * 32 + l] = v;
+                        }
+                        __syncthreads();
+                        if (tid < cnt) {
+                            double v = 0.0;
+                            for (int q = 0; q < p.nblk; ++q) v += gp[q * 32 + tid];
+                            sc[jb + tid] = (float)v;
+                        }
+                    }
+                    __syncthreads();
+                    const float* rb = p.RB + col;
+                    int j = 0;
+                    for (; j + 4 <= p.nb; j += 4) {
+                        const float c0 = sc[j], c1 = sc[j + 1], c2 = sc[j + 2], c3 = sc[j + 3];
+#pragma unroll
+                        for (int q = 0; q < kDotPerThread; ++q) {
+                            const int i = i0 + q * kDotThreads;
+                            if (i < N) {
+                                const float* e = rb + (int64_t)j * stride + i;
+                                const float b0 = e[0], b1 = e[stride], b2 = e[2 * stride], b3 = e[3 * stride];
+                                rv[q] = fmaf(-c0, b0, rv[q]);
+                                rv[q] = fmaf(-c1, b1, rv[q]);
+                                rv[q] = fmaf(-c2, b2, rv[q]);
+                                rv[q] = fmaf(-c3, b3, rv[q]);
+                            }
+                        }
+                    }
+                    for (; j < p.nb; ++j) {
+                        const float cj = sc[j];
+#pragma unroll
+                        for (int q = 0; q < kDotPerThread; ++q) {
+                            const int i = i0 + q * kDotThreads;
+                            if (i < N) rv[q] = fmaf(-cj, rb[(int64_t)j * stride + i], rv[q]);
+                        }
+                    }
+                    __syncthreads();   // sred, gp and sc are rewritten by the next pass
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kDotPerThread; ++q) {
+                const int i = i0 + q * kDotThreads;
+                if (i < N) {
+                    p.r[col + i] = rv[q];
+                    sr[i + (i >> 5)] = rv[q];
+                }
+            }
+            // z = P^{-1} r
+            float z[kDotPerThread];
+            if (p.rank > 0) {
+                const int k = p.rank, nb32 = (N + 31) / 32;
+                __syncthreads();
+                float* my = tile + w * 32 * 33;
+                for (int a0 = w; a0 < k; a0 += 32) {
+                    // lane l: the sum over rows of 32-row block b = l, l + 32, ..
+                    double v = 0.0;
+                    const float* La = p.L + (int64_t)a0 * N;
+                    for (int b0 = 0; b0 < nb32; b0 += 32) {
+#pragma unroll 16
+                        for (int e = 0; e < 32; ++e) {
+                            const int i = (b0 + e) * 32 + l;
+                            my[e * 33 + l] = i < N ? La[i] : 0.0f;
+                        }
+                        __syncwarp();
+                        const int b = b0 + l;
+                        if (b < nb32) {
+                            float acc = 0.0f;
+#pragma unroll 8
+                            for (int e = 0; e < 32; ++e)
+                                acc = fmaf(my[l * 33 + e], b * 32 + e < N ? sr[b * 33 + e] : 0.0f, acc);
+                            v += (double)acc;
+                        }
+                        __syncwarp();
+                    }
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if (l == 0) tv[a0] = v;
+                }
+                __syncthreads();
+                for (int a0 = w; a0 < k; a0 += 32) {
+                    double v = 0.0;
+                    for (int b = l; b < k; b += 32) v = fma(p.cinv[(int64_t)a0 * k + b], tv[b], v);
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if (l == 0) su[a0] = (float)v;
+                }
+                __syncthreads();
+                float acc[kDotPerThread];
+#pragma unroll
+                for (int q = 0; q < kDotPerThread; ++q) acc[q] = 0.0f;
+#pragma unroll 4
+                for (int a0 = 0; a0 < k; ++a0) {
+                    const float ua = su[a0];
+                    const float* La = p.L + (int64_t)a0 * N;
+#pragma unroll
+                    for (int q = 0; q < kDotPerThread; ++q) {
+                        const int i = i0 + q * kDotThreads;
+                        if (i < N) acc[q] = fmaf(La[i], ua, acc[q]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kDotPerThread; ++q) z[q] = p.inv_s2 * rv[q] - p.inv_s4 * acc[q];
+            } else {
+#pragma unroll
+                for (int q = 0; q < kDotPerThread; ++q) z[q] = rv[q];
+            }
+            // r^T z and beta
+            sh = sl = nh = nl = 0.0f;
+#pragma unroll
+            for (int q = 0; q < kDotPerThread; ++q) {
+                if (i0 + q * kDotThreads < N) {
+                    ff_add_prod(sh, sl, rv[q], z[q]);
+                    ff_add_prod(nh, nl, rv[q], rv[q]);
+                }
+            }
+            dots_reduce(sh, sl, nh, nl, t, sw + 8 * g, part + 3 * g, sync);
+            __syncthreads();
+            if (w == 0) {
+                scalar_column(SC_BETA, p.stable, part, p.nblk, p.R, p.st, c, l, p.k, p.tol, p.min_iter, p.ahist,
+                              p.bhist, p.rhist, p.nact, p.aflags);
+                if (l == 0) {
+                    s_beta = (float)S.beta;
+                    s_sg = (p.reorth == GP_REORTH_PINV) ? (float)(1.0 / sqrt(S.gamma))
+                                                        : (float)(S.rnorm > 0.0 ? 1.0 / S.rnorm : 0.0);
+                }
+            }
+            __syncthreads();
+            if (*active) {
+                // d = -z + beta d, this iterate's basis vectors, and the next MVM's copy of d
+                const float beta = s_beta, sg = s_sg;
+                int bad = 0;
+                float dn[kDotPerThread];
+#pragma unroll
+                for (int q = 0; q < kDotPerThread; ++q) {
+                    const int i = i0 + q * kDotThreads;
+                    if (i < N) {
+                        dn[q] = fmaf(beta, p.d[col + i], -z[q]);
+                        p.d[col + i] = dn[q];
+                        bad |= !(fabsf(dn[q]) <= 3.0e38f);
+                        if (p.reorth != GP_REORTH_NONE) {
+                            p.rho_k[col + i] = rv[q] * sg;
+                            if (p.reorth == GP_REORTH_PINV) p.zeta_k[col + i] = z[q] * sg;
+                        }
+                    }
+                }
+                if (p.v32) {
+                    bad = __syncthreads_or(bad);
+#pragma unroll
+                    for (int q = 0; q < kDotPerThread; ++q) {
+                        const int i = i0 + q * kDotThreads;
+                        if (i < N) p.v32[(int64_t)c * p.ld_v32 + i] = bad ? 0.0f : dn[q];
+                    }
+                    if (tid == 0) {
+                        p.outscale[c] = bad ? 0.0f : p.a2;
+                        if (bad) atomicCAS(p.err, 0, (int)DEV_NONFINITE);
+                    }
+                }
+            }
+        }
+    }
+    if (w == 0) scalar_ticket(p.st, p.R, l, p.nact);
+}
+
 int vec_grid(const Ctx* ctx, int64_t N) {
     int64_t g = (N + 255) / 256;
     const int64_t cap = 2 * (int64_t)(ctx->num_sms > 0 ? ctx->num_sms : 148);
@@ -550,6 +860,7 @@ int CgSolver::start(bool from_x, int k0) {
     const dim3 gcol((unsigned)vg, (unsigned)R);
     const size_t NR = (size_t)N * R;
     GPK_CUDA_TRY(cudaMemsetAsync(b.nact, 0, 2 * sizeof(int), s));
+    v_ready_op = nullptr;   // d is new
     if (from_x) {
         // the first start uses the solve's MVM; a restart the check MVM
         GPK_TRY(kop_apply(ctx, k0 > 0 ? *op_chk : op, U, R, b.Kd, N, true, s));
@@ -566,12 +877,71 @@ int CgSolver::start(bool from_x, int k0) {
     return flag_copy();
 }
 
+// The one-launch rest of an iteration: up to kTailMaxN rows, and as long as one CTA
+// reads its column's share (the factor twice, the bases) faster than thirteen launches
+// start: see the figures at cg_tail_kernel.
+bool CgSolver::tail_ok() const { return N <= kTailMaxN && N * (int64_t)(rank + 32) <= 600000; }
+
+int CgSolver::tail(const MvmParts& parts, KOp& mvm) {
+    TailParams p;
+    const size_t NR = (size_t)N * R;
+    p.N = (int)N;
+    p.R = R;
+    p.nblk = b.nblk_dot;
+    p.k = k;
+    p.nb = k - nb0 + 1;   // basis vectors r_0 .. r_k of this run
+    p.passes = passes;
+    p.reorth = reorth;
+    p.stable = stable;
+    p.rank = rank;
+    p.min_iter = o.min_iter;
+    p.tol = o.tol;
+    p.x = U;
+    p.r = b.r;
+    p.d = b.d;
+    p.Kd = parts.parts > 0 ? nullptr : b.Kd;
+    p.mv = parts;
+    p.ZB = reorth == GP_REORTH_PINV ? b.zeta : b.rho;
+    p.RB = b.rho;
+    const size_t slot = (size_t)p.nb;
+    p.rho_k = b.rho ? b.rho + slot * NR : nullptr;
+    p.zeta_k = b.zeta ? b.zeta + slot * NR : nullptr;
+    p.L = pc.L;
+    p.cinv = b.cinv;
+    p.inv_s2 = (float)(1.0 / hyp.noise);
+    p.inv_s4 = (float)(1.0 / (hyp.noise * hyp.noise));
+    p.st = b.st;
+    p.ahist = b.ahist;
+    p.bhist = b.bhist;
+    p.rhist = b.rhist;
+    p.nact = b.nact;
+    p.aflags = b.aflags;
+    const bool v32 = mvm.tp.engine == 1 && mvm.lay.fp32_pv;
+    p.v32 = v32 ? (float*)mvm.Vt : nullptr;
+    p.outscale = mvm.outscale;
+    p.ld_v32 = mvm.tp.Nc_pad;
+    p.a2 = mvm.a2;
+    p.err = ctx->dev_err;
+    v_ready_op = v32 ? &mvm : nullptr;
+    cg_tail_kernel<<<(unsigned)R, kTailThreads, tail_smem((int)N), s>>>(p);
+    GPK_TRY(launched(1));
+    ++k;
+    iters = k;
+    return flag_copy();
+}
+
 int CgSolver::iterate() {
     const dim3 gcol((unsigned)vg, (unsigned)R);
     const dim3 gdot((unsigned)b.nblk_dot, (unsigned)R);
     const size_t NR = (size_t)N * R;
     // Kd = Ktilde d
-    GPK_TRY(kop_apply(ctx, escalated ? *op_chk : refined ? *op_ref : op, b.d, R, b.Kd, N, true, s));
+    KOp& mvm = escalated ? *op_chk : refined ? *op_ref : op;
+    if (tail_ok()) {
+        MvmParts parts;
+        GPK_TRY(kop_apply(ctx, mvm, b.d, R, b.Kd, N, true, s, &parts, v_ready_op == &mvm));
+        return tail(parts, mvm);
+    }
+    GPK_TRY(kop_apply(ctx, mvm, b.d, R, b.Kd, N, true, s));
     GPK_TRY(dots(b.d, b.Kd, true));   // masked by the flags of the last scalar step
     GPK_TRY(scalar(SC_ALPHA, k));
     update_xr_kernel<<<gcol, 256, 0, s>>>(U, b.r, b.d, b.Kd, N, b.st);
@@ -659,6 +1029,9 @@ int CgSolver::setup(Ctx* c, WsCarver& wc, const gp_hyp_t* h, const float* X_, in
         }
     }
     wc_rest = wc;
+    if (tail_ok())
+        GPK_CUDA_TRY(cudaFuncSetAttribute(cg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tail_smem(kTailMaxN)));
     vg = vec_grid(ctx, N);
     k = nb0 = restarts = iters = 0;
     last_check = false;

@@ -155,9 +155,19 @@ bool tp_supported(int k_pad, int R_pad, int vsplit);
 int tp_rv(int R, int vsplit);   // rows of Vt per tile
 TcPlan tp_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad, int vsplit);
 size_t tp_partial_floats(const TcPlan& p);
+// An MVM result left as its partial sums, for a caller whose next kernel adds them
+// up itself: out[c][i] = outscale[c] sum_{q < parts} partial[(q R + c) ld + i]
+// + noise Vnoise[c][i], q in order.  parts = 0: the result was written.
+struct MvmParts {
+    const float* partial = nullptr;
+    const float* outscale = nullptr;
+    int parts = 0;
+    int64_t ld = 0;
+    float noise = 0.0f;
+};
 int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const MvmArgs& a, const CUtensorMap& tmA,
                    const CUtensorMap& tmB, const CUtensorMap& tmV, const float* outscale, float* partial,
-                   const uint32_t* mask, cudaStream_t s);
+                   const uint32_t* mask, cudaStream_t s, MvmParts* parts = nullptr);
 
 // SIMT FP32 engine (kmvm_simt.cu).  Scaled FP32 inputs with row stride dp.
 struct SimtPlan {
@@ -216,7 +226,10 @@ size_t kop_workspace(const Ctx* ctx, const gp_hyp_t* hyp, int64_t Nr, int64_t Nc
 int kop_prepare(Ctx* ctx, WsCarver& wc, KOp& op, const gp_hyp_t* hyp, const float* Xr, int64_t Nr,
                 const float* Xc, int64_t Nc, int R, int flags, cudaStream_t s);
 // out = K(Xr, Xc) V (+ sigma^2 V if add_noise); V: Nc x R (ld Nc), out: Nr x R (ld ld_out).
-int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_out, bool add_noise, cudaStream_t s);
+// parts: leave the result as partial sums where the engine has them (R <= 64; see MvmParts).
+// v_ready: the FP32 value product's copy of V (op.Vt) already holds it.
+int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_out, bool add_noise, cudaStream_t s,
+              MvmParts* parts = nullptr, bool v_ready = false);
 
 // Tensor-map helper (driver entry point fetched through the runtime).
 int encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uint64_t inner, uint64_t outer,
@@ -315,6 +328,9 @@ struct CgSolver {
     int finish(gp_cg_stats_t* stats);        // blocking: copy back, summarize
 
   private:
+    bool tail_ok() const;
+    int tail(const MvmParts& parts, KOp& mvm);
+    const KOp* v_ready_op = nullptr;   // operator whose FP32 copy of d the last tail kernel wrote
     int launched(int n);
     int flag_copy();
     int precond(const float* W, float* Z, bool masked);

@@ -849,7 +849,7 @@ size_t tp_partial_floats(const TcPlan& p) { return (size_t)p.n_split * p.rv * p.
 
 int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const MvmArgs& a, const CUtensorMap& tmA,
                    const CUtensorMap& tmB, const CUtensorMap& tmV, const float* outscale, float* partial,
-                   const uint32_t* mask, cudaStream_t s) {
+                   const uint32_t* mask, cudaStream_t s, MvmParts* parts) {
     TpParams prm;
     prm.n_ip = plan.n_it;
     prm.n_jt = plan.n_jt;
@@ -926,6 +926,14 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
     ctx->launches++;
     if (e != cudaSuccess) return GP_ERR_CUDA;
     if (!spv && plan.n_split == 1) return GP_OK;
+    if (parts) {
+        parts->partial = partial;
+        parts->outscale = outscale;
+        parts->parts = plan.n_split * (L.vsplit ? 2 : 1);
+        parts->ld = plan.Nr_pad;
+        parts->noise = a.noise + a.diag_coef;
+        return GP_OK;
+    }
     // splits times hi and lo rows (times the two column halves of the FP32 value product)
     return launch_split_reduce(ctx, partial, plan.n_split * (L.vsplit ? 2 : 1), plan.Nr_pad, a.Nr, a.R, a.R, outscale, 0.0f,
                                a.noise + a.diag_coef, a.Vnoise, a.Nc, a.out, a.ld_out, s);

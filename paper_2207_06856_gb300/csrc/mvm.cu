@@ -243,8 +243,10 @@ int kop_prepare(Ctx* ctx, WsCarver& wc, KOp& op, const gp_hyp_t* hyp, const floa
     return GP_OK;
 }
 
-int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_out, bool add_noise, cudaStream_t s) {
+int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_out, bool add_noise, cudaStream_t s,
+              MvmParts* parts, bool v_ready) {
     if (R > op.R_max) return GP_ERR_INVALID;
+    if (parts) parts->parts = 0;
     const int maxc = op.prec == GP_PREC_FP32 ? 32 : 64;
     for (int c0 = 0; c0 < R; c0 += maxc) {
         const int rc = (R - c0) < maxc ? (R - c0) : maxc;
@@ -276,16 +278,18 @@ int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_o
             pl.R_pad = ((rc + 15) / 16) * 16;
             if (pl.engine == 1) pl.rv = tp_rv(rc, op.lay.vsplit);
             const int vrows = pl.engine == 1 ? pl.rv : (op.lay.vsplit ? 2 : 1) * pl.R_pad;
-            GPK_TRY(launch_v_colmax(ctx, Vc, op.Nc, rc, op.cmax, s));
-            if (pl.engine == 1 && op.lay.fp32_pv) {
+            const bool fp32_pv = pl.engine == 1 && op.lay.fp32_pv;
+            if (!(fp32_pv && v_ready)) GPK_TRY(launch_v_colmax(ctx, Vc, op.Nc, rc, op.cmax, s));
+            if (fp32_pv) {
                 // FP32 value product: v in FP32 (4 rows, in the FP16 Vt buffer's space, which
                 // holds 2 x 16 FP16 rows), one TMA box of 128 columns x 4 rows per stage
-                GPK_TRY(launch_v_pack32(ctx, Vc, op.Nc, pl.Nc_pad, rc, op.cmax, op.a2, (float*)op.Vt, op.outscale,
-                                        s));
+                if (!v_ready)
+                    GPK_TRY(launch_v_pack32(ctx, Vc, op.Nc, pl.Nc_pad, rc, op.cmax, op.a2, (float*)op.Vt, op.outscale,
+                                            s));
                 GPK_TRY(encode_tmap_2d(&op.tmV, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, op.Vt, pl.Nc_pad, 4, pl.Nc_pad * 4,
                                        128, 4, CU_TENSOR_MAP_SWIZZLE_NONE));
                 GPK_TRY(launch_kmvm_tp(ctx, pl, op.lay, a, op.tmA, op.tmB, op.tmV, op.outscale, op.partial,
-                                       op.skip ? op.mask : nullptr, s));
+                                       op.skip ? op.mask : nullptr, s, parts));
                 continue;
             }
             GPK_TRY(launch_v_cast(ctx, op.prec, (op.flags & GP_MVM_SCALE_SQRT_N) ? 1 : 0, op.lay.vsplit, Vc, op.Nc,
@@ -298,7 +302,7 @@ int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_o
                 GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, (uint64_t)vrows, pl.Nc_pad * 2, 64, (uint32_t)pl.rv,
                                        CU_TENSOR_MAP_SWIZZLE_128B));
                 GPK_TRY(launch_kmvm_tp(ctx, pl, op.lay, a, op.tmA, op.tmB, op.tmV, op.outscale, op.partial,
-                                       op.skip ? op.mask : nullptr, s));
+                                       op.skip ? op.mask : nullptr, s, parts));
             } else {
                 GPK_TRY(encode_tmap_2d(&op.tmV, dt, op.Vt, pl.Nc_pad, (uint64_t)vrows, pl.Nc_pad * 2, 64, pl.R_pad,
                                        CU_TENSOR_MAP_SWIZZLE_128B));
