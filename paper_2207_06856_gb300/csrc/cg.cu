@@ -165,11 +165,9 @@ enum ScalarMode { SC_INIT = 0, SC_ALPHA = 1, SC_BETA = 2, SC_BNORM = 3 };
 
 // The scalar step of column c by one warp (lane l): merge the column's partials
 // (part: its nblk triples) in a fixed order, then the step of Alg. 1 / Alg. 2.
-__device__ void scalar_column(int mode, int stable, const double* part, int nblk, int R, ColState* __restrict__ st, int c,
-                              int l, int k, double tol, int min_iter, double* __restrict__ ahist,
-                              double* __restrict__ bhist, double* __restrict__ rhist, int* __restrict__ n_active,
-                              int* __restrict__ aflags) {
-    ColState& S = st[c];
+__device__ void scalar_column(int mode, int stable, const double* part, int nblk, int R, ColState& S, int c, int l,
+                              int k, double tol, int min_iter, double* __restrict__ ahist, double* __restrict__ bhist,
+                              double* __restrict__ rhist, int* __restrict__ n_active, int* __restrict__ aflags) {
     const bool act = (mode == SC_INIT || mode == SC_BNORM) ? true : (S.active != 0);
     if (act) {
         Lse acc{0.0, kEmptyExp};
@@ -250,6 +248,14 @@ __device__ void scalar_column(int mode, int stable, const double* part, int nblk
 // The last block of the grid to come here counts the active columns (n_active[2] is
 // its ticket, returned to 0 by that block).  One warp per block.
 __device__ void scalar_ticket(const ColState* __restrict__ st, int R, int l, int* __restrict__ n_active) {
+    if (gridDim.x == 1 && R == 1) {   // nobody else to wait for
+        if (l == 0) {
+            const int act = *(volatile const int*)&st[0].active != 0;
+            n_active[0] = act;
+            n_active[3] = act ? __float_as_int((float)*(volatile const double*)&st[0].relres) : 0;
+        }
+        return;
+    }
     int last = 0;
     if (l == 0) {
         __threadfence();
@@ -284,7 +290,7 @@ scalar_kernel(int mode, int stable, const double* __restrict__ part, int nblk, i
               int k, double tol, int min_iter, double* __restrict__ ahist, double* __restrict__ bhist,
               double* __restrict__ rhist, int* __restrict__ n_active, int* __restrict__ aflags) {
     const int c = blockIdx.x;
-    scalar_column(mode, stable, part + (int64_t)c * nblk * 3, nblk, R, st, c, threadIdx.x, k, tol, min_iter, ahist, bhist,
+    scalar_column(mode, stable, part + (int64_t)c * nblk * 3, nblk, R, st[c], c, threadIdx.x, k, tol, min_iter, ahist, bhist,
                   rhist, n_active, aflags);
     if (n_active) scalar_ticket(st, R, threadIdx.x, n_active);
 }
@@ -449,8 +455,9 @@ __global__ void reorth_update_kernel(const float* __restrict__ RB, int nb, int R
 // Everything between two MVMs is per column: one CTA per column runs it with block
 // barriers where the kernels above need a launch each (13 launches of 2-8 us for a
 // few thousand rows; one request of N = 2,000, rank 20, spent 115 us an iteration,
-// 7 of them in its MVM).  Thread t of group g (256 threads) owns elements
-// 2048 g + 256 q + t, q < 8, as in dots_kernel's chunks, with r and z in registers.
+// 7 of them in its MVM).  The vectors are in shared memory; element-wise steps
+// take element tid + 1024 m, the dots and Gram sums thread t of a 256-thread group
+// elements 2048 ch + 256 q + t of chunk ch, as in dots_kernel's and gram_kernel's blocks.
 // Every sum runs in the order of the kernels it stands for, so the results are the
 // same bit for bit: the split sums of the MVM, the float-float dots, the Gram
 // coefficients, the Woodbury apply (32-row blocks, FP64 across them).
@@ -478,15 +485,19 @@ struct TailParams {
     int* err;
 };
 
+// Vectors are stored with one word of padding per 32 elements.
+__host__ __device__ constexpr int tail_vec(int N) { return N + N / 32 + 33; }
 size_t tail_smem(int N) {
-    // part 16, gram sums 128, t 512 doubles; warp sums 32 float4; Gram 1024, coefficients 1024, u 512 floats;
-    // r with one word of padding per 32; a 32 x 33 staging tile per warp
+    // part 16, Gram sums 128, t 512 doubles; warp sums 32 float4; Gram 1024, coefficients 1024, u 512 floats;
+    // r and z; a 32 x 33 staging tile per warp, which holds d and Kd before it is needed
+    const size_t tile = 32 * 32 * 33, dk = 2 * (size_t)tail_vec(N);
     return (16 + 128 + 512) * sizeof(double) + 32 * sizeof(float4) +
-           (1024 + 1024 + 512 + (size_t)(N + N / 32 + 33) + 32 * 32 * 33) * sizeof(float);
+           (1024 + 1024 + 512 + 2 * (size_t)tail_vec(N) + (tile > dk ? tile : dk)) * sizeof(float);
 }
 
 __global__ void __launch_bounds__(kTailThreads, 1) cg_tail_kernel(const TailParams p) {
     extern __shared__ double tsm[];
+    const int N = p.N, vec = tail_vec(N);
     double* part = tsm;
     double* gp = part + 16;                                 // [4][32]
     double* tv = gp + 128;                                  // t = L^T r
@@ -494,246 +505,274 @@ __global__ void __launch_bounds__(kTailThreads, 1) cg_tail_kernel(const TailPara
     float* sred = reinterpret_cast<float*>(sw + 32);        // [4][8][32]
     float* sc = sred + 1024;                                // projection coefficients
     float* su = sc + 1024;                                  // u = C^{-1} t
-    float* tile = su + 512;                                 // [32 warps][32][33]
-    float* sr = tile + 32 * 32 * 33;                        // r, index i + i / 32
+    float* sr = su + 512;
+    float* sz = sr + vec;
+    float* tile = sz + vec;                                 // [32 warps][32][33]
+    float* sd = tile;
+    float* skd = tile + vec;
+    __shared__ ColState S;                                  // this column's state
     __shared__ float s_beta, s_sg;
     const int c = blockIdx.x, tid = threadIdx.x, g = tid >> 8, t = tid & 255, w = tid >> 5, l = tid & 31;
-    const int N = p.N;
     const int64_t col = (int64_t)c * N;
-    const int i0 = g * kDotChunk + t;                       // element q: i0 + 256 q
-    ColState& S = p.st[c];
-    volatile const int* active = &S.active;
-    volatile const double* alpha = &S.alpha;
     const auto sync = [] { __syncthreads(); };
+    const auto at = [](int i) { return i + (i >> 5); };
 
-    if (*active) {
-        // Kd (from the MVM's split sums where it left them), d^T K d and alpha
-        float kd[kDotPerThread], rv[kDotPerThread];
+    if (tid < (int)(sizeof(ColState) / 4)) ((int*)&S)[tid] = ((const int*)(p.st + c))[tid];
+    // d and Kd (from the MVM's split sums where it left them)
+    const float osc = p.Kd ? 0.0f : p.mv.outscale[c];
+    for (int i = tid; i < N; i += kTailThreads) {
+        const float dv = p.d[col + i];
+        float v;
+        if (p.Kd) {
+            v = p.Kd[col + i];
+        } else {
+            const float* q = p.mv.partial + (int64_t)c * p.mv.ld + i;
+            const int64_t step = (int64_t)p.R * p.mv.ld;
+            float sum = 0.0f;
+            int u = 0;
+            for (; u + 16 <= p.mv.parts; u += 16) {
+                float e[16];
+#pragma unroll
+                for (int x = 0; x < 16; ++x) e[x] = q[(u + x) * step];
+#pragma unroll
+                for (int x = 0; x < 16; ++x) sum += e[x];
+            }
+#pragma unroll 4
+            for (; u < p.mv.parts; ++u) sum += q[u * step];
+            v = sum * osc;
+            if (p.mv.noise != 0.0f) v = fmaf(p.mv.noise, dv, v);
+        }
+        sd[at(i)] = dv;
+        skd[at(i)] = v;
+    }
+    __syncthreads();
+    // float-float sums of a b and a^2 over this thread's elements of chunk g, then the group's
+    const auto dots = [&](const float* a, const float* b) {
         float sh = 0.0f, sl = 0.0f, nh = 0.0f, nl = 0.0f;
-        const float osc = p.Kd ? 0.0f : p.mv.outscale[c];
 #pragma unroll
         for (int q = 0; q < kDotPerThread; ++q) {
-            const int i = i0 + q * kDotThreads;
-            kd[q] = 0.0f;
+            const int i = g * kDotChunk + q * kDotThreads + t;
             if (i < N) {
-                const float dv = p.d[col + i];
-                if (p.Kd) {
-                    kd[q] = p.Kd[col + i];
-                } else {
-                    float sum = 0.0f;
-#pragma unroll 8
-                    for (int u = 0; u < p.mv.parts; ++u) sum += p.mv.partial[((int64_t)u * p.R + c) * p.mv.ld + i];
-                    float v = sum * osc;
-                    if (p.mv.noise != 0.0f) v = fmaf(p.mv.noise, dv, v);
-                    kd[q] = v;
-                }
-                ff_add_prod(sh, sl, dv, kd[q]);
-                ff_add_prod(nh, nl, dv, dv);
+                const float av = a[at(i)], bv = b[at(i)];
+                ff_add_prod(sh, sl, av, bv);
+                ff_add_prod(nh, nl, av, av);
             }
         }
         dots_reduce(sh, sl, nh, nl, t, sw + 8 * g, part + 3 * g, sync);
         __syncthreads();
+    };
+    if (S.active) {
+        dots(sd, skd);   // d^T K d
         if (w == 0)
-            scalar_column(SC_ALPHA, p.stable, part, p.nblk, p.R, p.st, c, l, p.k, p.tol, p.min_iter, p.ahist, p.bhist,
+            scalar_column(SC_ALPHA, p.stable, part, p.nblk, p.R, S, c, l, p.k, p.tol, p.min_iter, p.ahist, p.bhist,
                           p.rhist, p.nact, p.aflags);
         __syncthreads();
-        if (*active) {
-            const float a = (float)*alpha;
+    }
+    if (S.active) {
+        const float al = (float)S.alpha;
+        for (int i = tid; i < N; i += kTailThreads) {
+            p.x[col + i] = fmaf(al, sd[at(i)], p.x[col + i]);
+            sr[at(i)] = fmaf(al, skd[at(i)], p.r[col + i]);
+        }
+        __syncthreads();
+        // re-orthogonalisation: all coefficients, then the projection, per pass.  With one or two
+        // chunks the groups without one share the basis vectors.
+        const int64_t stride = (int64_t)p.R * N;
+        if (p.reorth != GP_REORTH_NONE) {
+            const int parts = p.nblk == 1 ? 4 : (p.nblk == 2 ? 2 : 1), nch = 4 / parts;
+            const int ch = g % nch, jp = g / nch, w8 = w & 7;
+            for (int pass = 0; pass < p.passes; ++pass) {
+                float rv[kDotPerThread];
 #pragma unroll
-            for (int q = 0; q < kDotPerThread; ++q) {
-                const int i = i0 + q * kDotThreads;
-                rv[q] = 0.0f;
-                if (i < N) {
-                    p.x[col + i] = fmaf(a, p.d[col + i], p.x[col + i]);
-                    rv[q] = fmaf(a, kd[q], p.r[col + i]);
+                for (int q = 0; q < kDotPerThread; ++q) {
+                    const int i = ch * kDotChunk + q * kDotThreads + t;
+                    rv[q] = i < N ? sr[at(i)] : 0.0f;
                 }
-            }
-            // re-orthogonalisation: all coefficients, then the projection, per pass
-            const int64_t stride = (int64_t)p.R * N;
-            if (p.reorth != GP_REORTH_NONE) {
-                for (int pass = 0; pass < p.passes; ++pass) {
-                    for (int jb = 0; jb < p.nb; jb += 32) {
-                        const int cnt = p.nb - jb < 32 ? p.nb - jb : 32;
-                        const float* zb = p.ZB + (int64_t)jb * stride + col;
-                        for (int j = 0; j < cnt; j += 4) {
-                            float av[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                for (int jb = 0; jb < p.nb; jb += 32) {
+                    const int cnt = p.nb - jb < 32 ? p.nb - jb : 32;
+                    const float* zb = p.ZB + (int64_t)jb * stride + col + ch * kDotChunk + t;
+                    for (int j = 4 * jp; j < cnt; j += 4 * parts) {
+                        float av[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-                            for (int q = 0; q < kDotPerThread; ++q) {
-                                const int i = i0 + q * kDotThreads;
-                                if (i < N) {
+                        for (int q = 0; q < kDotPerThread; ++q) {
+                            if (ch * kDotChunk + q * kDotThreads + t < N) {
 #pragma unroll
-                                    for (int u = 0; u < 4; ++u)
-                                        if (j + u < cnt) av[u] = fmaf(zb[(int64_t)(j + u) * stride + i], rv[q], av[u]);
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                for (int o = 16; o > 0; o >>= 1) av[u] += __shfl_xor_sync(0xffffffffu, av[u], o);
-                                if (l == 0 && j + u < cnt) sred[w * 32 + j + u] = av[u];
+                                for (int u = 0; u < 4; ++u)
+                                    if (j + u < cnt)
+                                        av[u] = fmaf(zb[(int64_t)(j + u) * stride + q * kDotThreads], rv[q], av[u]);
                             }
                         }
-                        __syncthreads();
-                        if (w < p.nblk && l < cnt) {   // warp w: chunk w's 8 warp sums
-                            double v = 0.0;
-                            for (int q = 0; q < 8; ++q) v += (double)sred[(8 * w + q) * 32 + l];
-                            gp[w * 32 + l] = v;
-                        }
-                        __syncthreads();
-                        if (tid < cnt) {
-                            double v = 0.0;
-                            for (int q = 0; q < p.nblk; ++q) v += gp[q * 32 + tid];
-                            sc[jb + tid] = (float)v;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            for (int o = 16; o > 0; o >>= 1) av[u] += __shfl_xor_sync(0xffffffffu, av[u], o);
+                            if (l == 0 && j + u < cnt) sred[(ch * 8 + w8) * 32 + j + u] = av[u];
                         }
                     }
                     __syncthreads();
-                    const float* rb = p.RB + col;
+                    if (w < p.nblk && l < cnt) {   // warp w: chunk w's 8 warp sums
+                        double v = 0.0;
+                        for (int q = 0; q < 8; ++q) v += (double)sred[(8 * w + q) * 32 + l];
+                        gp[w * 32 + l] = v;
+                    }
+                    __syncthreads();
+                    if (tid < cnt) {
+                        double v = 0.0;
+                        for (int q = 0; q < p.nblk; ++q) v += gp[q * 32 + tid];
+                        sc[jb + tid] = (float)v;
+                    }
+                }
+                __syncthreads();
+                for (int i = tid; i < N; i += 2 * kTailThreads) {   // two elements, eight loads of each in flight
+                    const int i2 = i + kTailThreads;
+                    const bool two = i2 < N;
+                    const float* e0 = p.RB + col + i;
+                    const float* e1 = two ? e0 + kTailThreads : e0;
+                    float v0 = sr[at(i)], v1 = two ? sr[at(i2)] : 0.0f;
                     int j = 0;
-                    for (; j + 4 <= p.nb; j += 4) {
-                        const float c0 = sc[j], c1 = sc[j + 1], c2 = sc[j + 2], c3 = sc[j + 3];
+                    for (; j + 8 <= p.nb; j += 8) {
+                        float b0[8], b1[8];
 #pragma unroll
-                        for (int q = 0; q < kDotPerThread; ++q) {
-                            const int i = i0 + q * kDotThreads;
-                            if (i < N) {
-                                const float* e = rb + (int64_t)j * stride + i;
-                                const float b0 = e[0], b1 = e[stride], b2 = e[2 * stride], b3 = e[3 * stride];
-                                rv[q] = fmaf(-c0, b0, rv[q]);
-                                rv[q] = fmaf(-c1, b1, rv[q]);
-                                rv[q] = fmaf(-c2, b2, rv[q]);
-                                rv[q] = fmaf(-c3, b3, rv[q]);
-                            }
+                        for (int u = 0; u < 8; ++u) {
+                            b0[u] = e0[(int64_t)(j + u) * stride];
+                            b1[u] = e1[(int64_t)(j + u) * stride];
+                        }
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            v0 = fmaf(-sc[j + u], b0[u], v0);
+                            v1 = fmaf(-sc[j + u], b1[u], v1);
                         }
                     }
-                    for (; j < p.nb; ++j) {
-                        const float cj = sc[j];
-#pragma unroll
-                        for (int q = 0; q < kDotPerThread; ++q) {
-                            const int i = i0 + q * kDotThreads;
-                            if (i < N) rv[q] = fmaf(-cj, rb[(int64_t)j * stride + i], rv[q]);
-                        }
-                    }
-                    __syncthreads();   // sred, gp and sc are rewritten by the next pass
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < kDotPerThread; ++q) {
-                const int i = i0 + q * kDotThreads;
-                if (i < N) {
-                    p.r[col + i] = rv[q];
-                    sr[i + (i >> 5)] = rv[q];
-                }
-            }
-            // z = P^{-1} r
-            float z[kDotPerThread];
-            if (p.rank > 0) {
-                const int k = p.rank, nb32 = (N + 31) / 32;
-                __syncthreads();
-                float* my = tile + w * 32 * 33;
-                for (int a0 = w; a0 < k; a0 += 32) {
-                    // lane l: the sum over rows of 32-row block b = l, l + 32, ..
-                    double v = 0.0;
-                    const float* La = p.L + (int64_t)a0 * N;
-                    for (int b0 = 0; b0 < nb32; b0 += 32) {
-#pragma unroll 16
-                        for (int e = 0; e < 32; ++e) {
-                            const int i = (b0 + e) * 32 + l;
-                            my[e * 33 + l] = i < N ? La[i] : 0.0f;
-                        }
-                        __syncwarp();
-                        const int b = b0 + l;
-                        if (b < nb32) {
-                            float acc = 0.0f;
-#pragma unroll 8
-                            for (int e = 0; e < 32; ++e)
-                                acc = fmaf(my[l * 33 + e], b * 32 + e < N ? sr[b * 33 + e] : 0.0f, acc);
-                            v += (double)acc;
-                        }
-                        __syncwarp();
-                    }
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (l == 0) tv[a0] = v;
-                }
-                __syncthreads();
-                for (int a0 = w; a0 < k; a0 += 32) {
-                    double v = 0.0;
-                    for (int b = l; b < k; b += 32) v = fma(p.cinv[(int64_t)a0 * k + b], tv[b], v);
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (l == 0) su[a0] = (float)v;
-                }
-                __syncthreads();
-                float acc[kDotPerThread];
-#pragma unroll
-                for (int q = 0; q < kDotPerThread; ++q) acc[q] = 0.0f;
 #pragma unroll 4
-                for (int a0 = 0; a0 < k; ++a0) {
-                    const float ua = su[a0];
-                    const float* La = p.L + (int64_t)a0 * N;
-#pragma unroll
-                    for (int q = 0; q < kDotPerThread; ++q) {
-                        const int i = i0 + q * kDotThreads;
-                        if (i < N) acc[q] = fmaf(La[i], ua, acc[q]);
+                    for (; j < p.nb; ++j) {
+                        v0 = fmaf(-sc[j], e0[(int64_t)j * stride], v0);
+                        v1 = fmaf(-sc[j], e1[(int64_t)j * stride], v1);
                     }
+                    sr[at(i)] = v0;
+                    if (two) sr[at(i2)] = v1;
                 }
-#pragma unroll
-                for (int q = 0; q < kDotPerThread; ++q) z[q] = p.inv_s2 * rv[q] - p.inv_s4 * acc[q];
-            } else {
-#pragma unroll
-                for (int q = 0; q < kDotPerThread; ++q) z[q] = rv[q];
+                __syncthreads();   // r is complete; sred, gp and sc may be rewritten
             }
-            // r^T z and beta
-            sh = sl = nh = nl = 0.0f;
+        }
+        // z = P^{-1} r
+        if (p.rank > 0) {
+            const int k = p.rank, nb32 = (N + 31) / 32;
+            // t = L^T r.  d and Kd give their place to the staging tiles here (last read before a barrier).
+            float* my = tile + w * 32 * 33;
+            for (int a0 = w; a0 < k; a0 += 32) {
+                // lane l: the sum over rows of 32-row blocks b = l, l + 32, ..
+                double v = 0.0;
+                const float* La = p.L + (int64_t)a0 * N;
+                for (int b0 = 0; b0 < nb32; b0 += 32) {
+                    float e[32];
 #pragma unroll
-            for (int q = 0; q < kDotPerThread; ++q) {
-                if (i0 + q * kDotThreads < N) {
-                    ff_add_prod(sh, sl, rv[q], z[q]);
-                    ff_add_prod(nh, nl, rv[q], rv[q]);
+                    for (int x = 0; x < 32; ++x) {
+                        const int i = (b0 + x) * 32 + l;
+                        e[x] = i < N ? La[i] : 0.0f;
+                    }
+#pragma unroll
+                    for (int x = 0; x < 32; ++x) my[x * 33 + l] = e[x];
+                    __syncwarp();
+                    const int b = b0 + l;
+                    if (b < nb32) {
+                        float acc = 0.0f;
+#pragma unroll 8
+                        for (int x = 0; x < 32; ++x)
+                            acc = fmaf(my[l * 33 + x], b * 32 + x < N ? sr[b * 33 + x] : 0.0f, acc);
+                        v += (double)acc;
+                    }
+                    __syncwarp();
                 }
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (l == 0) tv[a0] = v;
             }
-            dots_reduce(sh, sl, nh, nl, t, sw + 8 * g, part + 3 * g, sync);
             __syncthreads();
-            if (w == 0) {
-                scalar_column(SC_BETA, p.stable, part, p.nblk, p.R, p.st, c, l, p.k, p.tol, p.min_iter, p.ahist,
-                              p.bhist, p.rhist, p.nact, p.aflags);
-                if (l == 0) {
-                    s_beta = (float)S.beta;
-                    s_sg = (p.reorth == GP_REORTH_PINV) ? (float)(1.0 / sqrt(S.gamma))
-                                                        : (float)(S.rnorm > 0.0 ? 1.0 / S.rnorm : 0.0);
-                }
+            for (int a0 = w; a0 < k; a0 += 32) {
+                double v = 0.0;
+#pragma unroll 4
+                for (int b = l; b < k; b += 32) v = fma(p.cinv[(int64_t)a0 * k + b], tv[b], v);
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (l == 0) su[a0] = (float)v;
             }
             __syncthreads();
-            if (*active) {
-                // d = -z + beta d, this iterate's basis vectors, and the next MVM's copy of d
-                const float beta = s_beta, sg = s_sg;
-                int bad = 0;
-                float dn[kDotPerThread];
+            for (int i = tid; i < N; i += 2 * kTailThreads) {
+                const int i2 = i + kTailThreads;
+                const bool two = i2 < N;
+                const float* e0 = p.L + i;
+                const float* e1 = two ? e0 + kTailThreads : e0;
+                float a0 = 0.0f, a1 = 0.0f;
+                int a = 0;
+                for (; a + 8 <= k; a += 8) {
+                    float b0[8], b1[8];
 #pragma unroll
-                for (int q = 0; q < kDotPerThread; ++q) {
-                    const int i = i0 + q * kDotThreads;
-                    if (i < N) {
-                        dn[q] = fmaf(beta, p.d[col + i], -z[q]);
-                        p.d[col + i] = dn[q];
-                        bad |= !(fabsf(dn[q]) <= 3.0e38f);
-                        if (p.reorth != GP_REORTH_NONE) {
-                            p.rho_k[col + i] = rv[q] * sg;
-                            if (p.reorth == GP_REORTH_PINV) p.zeta_k[col + i] = z[q] * sg;
-                        }
+                    for (int u = 0; u < 8; ++u) {
+                        b0[u] = e0[(int64_t)(a + u) * N];
+                        b1[u] = e1[(int64_t)(a + u) * N];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        a0 = fmaf(b0[u], su[a + u], a0);
+                        a1 = fmaf(b1[u], su[a + u], a1);
                     }
                 }
-                if (p.v32) {
-                    bad = __syncthreads_or(bad);
-#pragma unroll
-                    for (int q = 0; q < kDotPerThread; ++q) {
-                        const int i = i0 + q * kDotThreads;
-                        if (i < N) p.v32[(int64_t)c * p.ld_v32 + i] = bad ? 0.0f : dn[q];
-                    }
-                    if (tid == 0) {
-                        p.outscale[c] = bad ? 0.0f : p.a2;
-                        if (bad) atomicCAS(p.err, 0, (int)DEV_NONFINITE);
-                    }
+#pragma unroll 4
+                for (; a < k; ++a) {
+                    a0 = fmaf(e0[(int64_t)a * N], su[a], a0);
+                    a1 = fmaf(e1[(int64_t)a * N], su[a], a1);
+                }
+                sz[at(i)] = p.inv_s2 * sr[at(i)] - p.inv_s4 * a0;
+                if (two) sz[at(i2)] = p.inv_s2 * sr[at(i2)] - p.inv_s4 * a1;
+            }
+        } else {
+            for (int i = tid; i < N; i += kTailThreads) sz[at(i)] = sr[at(i)];
+        }
+        __syncthreads();
+        dots(sr, sz);   // r^T z
+        if (w == 0) {
+            scalar_column(SC_BETA, p.stable, part, p.nblk, p.R, S, c, l, p.k, p.tol, p.min_iter, p.ahist, p.bhist,
+                          p.rhist, p.nact, p.aflags);
+            if (l == 0) {
+                s_beta = (float)S.beta;
+                s_sg = (p.reorth == GP_REORTH_PINV) ? (float)(1.0 / sqrt(S.gamma))
+                                                    : (float)(S.rnorm > 0.0 ? 1.0 / S.rnorm : 0.0);
+            }
+        } else {
+            for (int i = tid - 32; i < N; i += kTailThreads - 32) p.r[col + i] = sr[at(i)];
+        }
+        __syncthreads();
+        if (S.active) {
+            // d = -z + beta d, this iterate's basis vectors, and the next MVM's copy of d
+            const float beta = s_beta, sg = s_sg;
+            int bad = 0;
+            for (int i = tid; i < N; i += kTailThreads) {
+                const float zi = sz[at(i)];
+                const float dn = fmaf(beta, p.d[col + i], -zi);
+                p.d[col + i] = dn;
+                bad |= !(fabsf(dn) <= 3.0e38f);
+                if (p.v32) p.v32[(int64_t)c * p.ld_v32 + i] = dn;
+                if (p.reorth != GP_REORTH_NONE) {
+                    p.rho_k[col + i] = sr[at(i)] * sg;
+                    if (p.reorth == GP_REORTH_PINV) p.zeta_k[col + i] = zi * sg;
+                }
+            }
+            if (p.v32) {
+                bad = __syncthreads_or(bad);
+                if (bad)   // as launch_v_pack32: a column with a non-finite value is zero
+                    for (int i = tid; i < N; i += kTailThreads) p.v32[(int64_t)c * p.ld_v32 + i] = 0.0f;
+                if (tid == 0) {
+                    p.outscale[c] = bad ? 0.0f : p.a2;
+                    if (bad) atomicCAS(p.err, 0, (int)DEV_NONFINITE);
                 }
             }
         }
     }
-    if (w == 0) scalar_ticket(p.st, p.R, l, p.nact);
+    // the state goes back (its last writes were before a barrier), then the count
+    if (w == 0) {
+        __syncwarp();
+        for (int e = l; e < (int)(sizeof(ColState) / 4); e += 32) ((int*)(p.st + c))[e] = ((const int*)&S)[e];
+        __threadfence();
+        __syncwarp();
+        scalar_ticket(p.st, p.R, l, p.nact);
+    }
 }
 
 int vec_grid(const Ctx* ctx, int64_t N) {
