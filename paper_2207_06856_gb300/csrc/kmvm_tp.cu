@@ -80,6 +80,8 @@ struct TpSmem {
     uint32_t total;   // dynamic shared memory to request (includes 1 KB alignment slack)
 };
 
+constexpr uint32_t kOneCtaSmem = 116u << 10;
+
 __host__ __device__ inline TpSmem tp_smem(int k_pad, int rv) {
     TpSmem m;
     m.xbytes = (uint32_t)kBM * (uint32_t)k_pad * 2u;
@@ -90,6 +92,9 @@ __host__ __device__ inline TpSmem tp_smem(int k_pad, int rv) {
     for (int s = kMaxStages; s >= 2; --s)
         if (fixed + (uint32_t)s * m.stage_bytes <= (uint32_t)kMaxSmemBytes - 512u) { m.stages = s; break; }
     m.total = fixed + (uint32_t)m.stages * m.stage_bytes;
+    // More than half of the SM's shared memory: a CTA allocates all of TMEM, so a second one
+    // on its SM (another stream's) would hold threads and registers only to wait for it.
+    if (m.total < kOneCtaSmem) m.total = kOneCtaSmem;
     return m;
 }
 

@@ -67,6 +67,7 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity, 
     const long long lim = (long long)(limit_ns * 2ull);
     while (true) {
         if (mbar_try_wait_hint(bar, parity, 20000u)) return true;
+        // a last look: the time may have passed with this warp switched out
         if (clock64() - t0 > lim) return mbar_try_wait(bar, parity);
     }
 }
@@ -98,6 +99,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
 
 // ---- named barriers (id 0 is __syncthreads) -----------------------------------
 __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {
+    __syncwarp();   // the warp arrives as one
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 // Arrival of a warp that goes on.  A warp whose bounded wait ran out (ok = false) no
