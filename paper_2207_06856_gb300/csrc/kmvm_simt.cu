@@ -15,7 +15,13 @@
 // IEEE round-to-nearest operations per instruction): a row's squared distance
 // as two interleaved partial sums over even and odd dimensions, and its
 // accumulators as pairs of adjacent output columns.  Shared memory holds the
-// negated column inputs so the difference is one packed add.
+// negated column inputs so the difference is one packed add.  Two columns at a time, so
+// that one column's shared-memory reads and exponentials run beside the other's FMAs, and
+// no test of the column count inside (the accumulators in use are compiled in); each
+// accumulator still takes its columns in order.  Bound by the FMA pipe: 36 FP32 operations a
+// pair at d = 8, R = 17 are 1,030 us at N = 32,768; 2,262 us with one column at a time and
+// the tests (FMA pipe 45 % busy, waiting for shared memory), 1,512 without the tests,
+// 1,370 as it is (three columns at a time 1,335, four 1,398, at 20 to 50 more registers).
 #include "gpk_internal.cuh"
 #include "kfun.cuh"
 
@@ -26,6 +32,57 @@ namespace {
 constexpr int kSimtThreads = 128;
 constexpr int kSimtRows = 2 * kSimtThreads;
 constexpr int kSimtTile = 64;
+constexpr int kSimtCols = 2;
+
+// q += |x + (-x_j)|^2 over four dimensions (even and odd ones summed apart).
+__device__ __forceinline__ void simt_dist(float2 xa, float2 xb, const float4& nx, float2& q) {
+    const float2 da = __fadd2_rn(xa, make_float2(nx.x, nx.y)), db = __fadd2_rn(xb, make_float2(nx.z, nx.w));
+    q = __ffma2_rn(da, da, q);
+    q = __ffma2_rn(db, db, q);
+}
+// a, b += k v over four columns of V.
+__device__ __forceinline__ void simt_acc(float k, const float4& v, float2& a, float2& b) {
+    const float2 kk = make_float2(k, k);
+    a = __ffma2_rn(kk, make_float2(v.x, v.y), a);
+    b = __ffma2_rn(kk, make_float2(v.z, v.w), b);
+}
+
+// C columns for the thread's two rows.  RPM = R rounded up to 4: every group of four columns
+// of V is in use.
+template <int KIND, int DPM, int RPM, int C>
+__device__ __forceinline__ void simt_columns(const float (*sx)[DPM + 4], const float (*sv)[RPM + 4], int dp,
+                                             const float2 (&x0)[DPM / 2], const float2 (&x1)[DPM / 2],
+                                             float2 (&acc0)[RPM / 2], float2 (&acc1)[RPM / 2]) {
+    float2 q0[C], q1[C];
+#pragma unroll
+    for (int u = 0; u < C; ++u) q0[u] = q1[u] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < DPM; k += 4) {
+        if (k < dp) {
+#pragma unroll
+            for (int u = 0; u < C; ++u) {
+                const float4 nx = *reinterpret_cast<const float4*>(&sx[u][k]);   // broadcast
+                simt_dist(x0[k / 2], x0[k / 2 + 1], nx, q0[u]);
+                simt_dist(x1[k / 2], x1[k / 2 + 1], nx, q1[u]);
+            }
+        }
+    }
+    float k0[C], k1[C];
+#pragma unroll
+    for (int u = 0; u < C; ++u) {
+        k0[u] = kernel_from_s<KIND>(-(q0[u].x + q0[u].y));
+        k1[u] = kernel_from_s<KIND>(-(q1[u].x + q1[u].y));
+    }
+#pragma unroll
+    for (int c = 0; c < RPM; c += 4) {
+#pragma unroll
+        for (int u = 0; u < C; ++u) {
+            const float4 v4 = *reinterpret_cast<const float4*>(&sv[u][c]);   // broadcast
+            simt_acc(k0[u], v4, acc0[c / 2], acc0[c / 2 + 1]);
+            simt_acc(k1[u], v4, acc1[c / 2], acc1[c / 2 + 1]);
+        }
+    }
+}
 
 template <int KIND, int DPM, int RPM>
 __global__ void __launch_bounds__(kSimtThreads)
@@ -66,36 +123,11 @@ kmvm_simt_kernel(const float* __restrict__ Xr, const float* __restrict__ Xc, con
         }
         __syncthreads();
         const int jn = (int)((Nc - jb) < kSimtTile ? (Nc - jb) : kSimtTile);
-        for (int jj = 0; jj < jn; ++jj) {
-            float2 q0 = make_float2(0.0f, 0.0f), q1 = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int k = 0; k < DPM; k += 4) {
-                if (k < dp) {
-                    const float4 x4 = *reinterpret_cast<const float4*>(&sx[jj][k]);   // broadcast
-                    const float2 xa = make_float2(x4.x, x4.y), xb = make_float2(x4.z, x4.w);
-                    const float2 d0a = __fadd2_rn(x0[k / 2], xa), d0b = __fadd2_rn(x0[k / 2 + 1], xb);
-                    const float2 d1a = __fadd2_rn(x1[k / 2], xa), d1b = __fadd2_rn(x1[k / 2 + 1], xb);
-                    q0 = __ffma2_rn(d0a, d0a, q0);
-                    q1 = __ffma2_rn(d1a, d1a, q1);
-                    q0 = __ffma2_rn(d0b, d0b, q0);
-                    q1 = __ffma2_rn(d1b, d1b, q1);
-                }
-            }
-            const float k0 = kernel_from_s<KIND>(-(q0.x + q0.y));
-            const float k1 = kernel_from_s<KIND>(-(q1.x + q1.y));
-            const float2 kk0 = make_float2(k0, k0), kk1 = make_float2(k1, k1);
-#pragma unroll
-            for (int c = 0; c < RPM; c += 4) {
-                if (c < R) {
-                    const float4 v4 = *reinterpret_cast<const float4*>(&sv[jj][c]);   // broadcast
-                    const float2 va = make_float2(v4.x, v4.y), vb = make_float2(v4.z, v4.w);
-                    acc0[c / 2] = __ffma2_rn(kk0, va, acc0[c / 2]);
-                    acc1[c / 2] = __ffma2_rn(kk1, va, acc1[c / 2]);
-                    acc0[c / 2 + 1] = __ffma2_rn(kk0, vb, acc0[c / 2 + 1]);
-                    acc1[c / 2 + 1] = __ffma2_rn(kk1, vb, acc1[c / 2 + 1]);
-                }
-            }
-        }
+        int jj = 0;
+        for (; jj + kSimtCols <= jn; jj += kSimtCols)
+            simt_columns<KIND, DPM, RPM, kSimtCols>(&sx[jj], &sv[jj], dp, x0, x1, acc0, acc1);
+#pragma unroll 1
+        for (; jj < jn; ++jj) simt_columns<KIND, DPM, RPM, 1>(&sx[jj], &sv[jj], dp, x0, x1, acc0, acc1);
         __syncthreads();
     }
 #pragma unroll
