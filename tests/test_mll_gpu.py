@@ -284,3 +284,22 @@ def test_vjp_tensor_core_differentiation_inputs_n16384(ctx):
     ref, refX = C.quad_form_grad(w.X, oh, U.T, V.T, wrt_X=True)
     assert _rel(g, ref) <= 1e-2, (g, ref)
     assert _rel(gX.cpu().numpy(), refX) <= 1e-2
+
+
+@pytest.mark.parametrize("kern", [0, 3])
+@pytest.mark.parametrize("shape", [(2, 1, 1), (127, 7, 2), (128, 8, 16), (129, 15, 17), (257, 16, 16), (255, 20, 31)])
+def test_vjp_tensor_core_tile_edges(ctx, kern, shape):
+    """Rows at the edges of the 128-row tiles and 64-column slots, 2 (d + 1) output columns
+    at the edges of their groups of 16, right-hand sides at the edges of 16.  Operands and
+    W' rounded to FP16 (2^-11 each, four roundings): <= 1e-2 relative in the vector norm,
+    as for the other shapes."""
+    from paper_2207_06856_gb300 import gpk
+    N, d, R = shape
+    X, V, _, ls, a2, s2 = workloads.random_problem(N, d, R, seed=N + 7 * d, kernel=kern)
+    U = np.random.default_rng(N + 1).standard_normal((R, N)).astype(np.float32)
+    hyp = gpk.Hyper(kern, ls, a2, s2)
+    g, gX = gpk.kmvm_vjp(ctx, hyp, _dev(X), _dev(U), _dev(V), want_X=True, precision="fp16")
+    ctx.check()
+    ref, refX = O.quad_form_grad(X, O.Hyp(KNAME[kern], ls, a2, s2), U.T, V.T, wrt_X=True)
+    assert _rel(g, ref) <= 1e-2, (g, ref)
+    assert _rel(gX.cpu().numpy(), refX) <= 1e-2
