@@ -122,13 +122,12 @@ extern "C" {
                                        done by the epilogue threads in FP32 FMAs
                                        (v as hi + lo), instead of rounding P to
                                        FP16 for a tensor-core product whose
-                                       M = 128 rows would hold 1..4 right-hand
+                                       16 columns would hold 1..4 right-hand
                                        sides.  For the single-column solves of
                                        serving.  Other shapes: GP_ERR_UNSUPPORTED. */
 #define GP_MVM_ONE_TILE     0x4000  /* tensor-core MVM on the one-row-tile engine
                                        (P V with M = 128 rows, N = R) instead of
-                                       the default pair engine (transposed
-                                       V^T P^T, N = 256 rows); for comparison     */
+                                       the default pair engine; for comparison     */
 
 /* GP hyperparameters theta = (l_1..l_d, a^2, sigma^2)   (Sec. 2.2, Eq. mvm) */
 typedef struct {
