@@ -72,7 +72,7 @@ RELAX_RESID = 30.0 * TOL
 # keyed by the launch it was captured on (kernel, precision, N, R, flags); the
 # roofline reports it only for that exact launch and null otherwise.
 KMVM_TRAFFIC_BYTES = {("rbf", "fp16", 65536, 17, 0): 10.522624e6 + 0.0,
-                      ("rbf", "fp16", 65536, 17, 0x8000 | 0x200): 16.880896e6 + 11.435264e6}   # PSPLIT | XSPLIT
+                      ("rbf", "fp16", 65536, 17, 0x8000 | 0x200): 14.721792e6 + 0.005888e6}   # PSPLIT | XSPLIT
 
 
 def _peaks_file():
