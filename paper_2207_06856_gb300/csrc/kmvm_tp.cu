@@ -127,7 +127,7 @@ struct TpBarriers {
     // S and P buffers, [2 x ring slot + row tile]
     uint64_t s_full[kMaxBufs];
     uint64_t p_empty[kMaxBufs]; // P consumed by its value product (and, in place, S may be rewritten)
-    uint64_t o_full[2];         // per row tile
+    uint64_t o_full[2];         // per row tile, once per item with an evaluated tile
     uint64_t xi_full[2];
     uint64_t xi_empty[2];
     uint64_t drain[4];          // per issuing warp
@@ -369,7 +369,10 @@ __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sS
             if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
             acc = 1;
         }
-        if (si.ok) ptx::mma_commit_elect(&bars.o_full[w]);
+        // An item without an evaluated tile has no O.  One with tiles meets the epilogue at
+        // bar_p_full, after the epilogue's wait for the last such item's O: the issuer is
+        // never two phases of o_full ahead, where the wait's parity would repeat.
+        if (acc && si.ok) ptx::mma_commit_elect(&bars.o_full[w]);
     }
     const uint32_t dr = MODE == kInPlace ? 2u + w : w;
     ptx::mma_commit_elect(&bars.drain[dr]);
@@ -484,10 +487,10 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
     const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
     const int row = wq * 32 + lane;                   // row within the tile
     uint32_t b = 0, ph = 0;                           // buffer ring slot and its fill parity
-    int ic = 0;
+    uint32_t oph = 0;                                 // parity of the next O: items with an evaluated tile only
     bool ok = true;
 #pragma unroll 1
-    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
         const int it = 2 * ip + tl;   // this warpgroup's row tile
@@ -567,7 +570,10 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
             any = true;
         }
         // O read-out: lanes are rows of the tile; this warpgroup's half of the right-hand sides.
-        ok = ok && warp_wait(&bars.o_full[tl], ic & 1, p.limit_ns);
+        if (any) {
+            ok = ok && warp_wait(&bars.o_full[tl], oph, p.limit_ns);
+            oph ^= 1u;
+        }
         ptx::tc_fence_after();
         const int half = (p.nrhs + 1) >> 1;
         const int c0 = ch * half, c1 = ch ? p.nrhs : half;

@@ -534,3 +534,29 @@ def test_fp32_few_rows_many_splits(ctx, Nr, R):
     ref = _ref(Xr, V, 1, ls, a2, s2, Xc=X, add_noise=False)
     mag = _ref(Xr, np.abs(V), 1, ls, a2, s2, Xc=X, add_noise=False)
     assert np.all(np.abs(got - ref) <= TOL["fp32"] * mag)
+
+
+@pytest.mark.parametrize("square", [True, False])
+@pytest.mark.parametrize("flags_name", ["", "MVM_PSPLIT"])
+@pytest.mark.parametrize("R", [1, 17, 64])
+def test_skip_tiles_runs_of_empty_items(ctx, R, flags_name, square):
+    """Many work items per CTA, most of them without an evaluated tile, in runs and at
+    the end: 64 compact clusters 20 lengthscales apart, 625 points each (313 column tiles,
+    157 row-tile pairs; a pair meets one or two of a dozen column ranges), and the columns
+    of four clusters alone (whole row-tile pairs without a tile).  Skipped tiles hold
+    kernel values that round to zero, so the result is bit-identical."""
+    from paper_2207_06856_gb300 import gpk
+    g = (np.arange(8) - 3.5) * 20.0
+    X = _clusters(625, [np.array([a, b, 0.0]) for a in g for b in g], 0.05, seed=51, ragged=37)
+    Xc = X if square else np.ascontiguousarray(X[20 * 625:24 * 625])
+    V = np.random.default_rng(52).standard_normal((R, Xc.shape[0])).astype(np.float32)
+    ls = np.ones(3, np.float32)
+    base = getattr(gpk, flags_name) if flags_name else 0
+    arg = {} if square else {"Xc": Xc, "add_noise": False}
+    a = _run(ctx, X, V, 0, ls, 1.0, 0.05, "fp16", flags=base, **arg)
+    b = _run(ctx, X, V, 0, ls, 1.0, 0.05, "fp16", flags=base | gpk.MVM_SKIP_TILES, **arg)
+    assert np.array_equal(a, b)
+    dev = torch.device("cuda:0")
+    ev, tot = gpk.kmvm_tile_count(ctx, gpk.Hyper(0, ls, 1.0, 0.05), torch.from_numpy(X).to(dev),
+                                  None if square else torch.from_numpy(Xc).to(dev), flags=base | gpk.MVM_SKIP_TILES)
+    assert 0 < ev < 0.15 * tot, (ev, tot)
