@@ -455,12 +455,14 @@ __global__ void reorth_update_kernel(const float* __restrict__ RB, int nb, int R
 // Everything between two MVMs is per column: one CTA per column runs it with block
 // barriers where the kernels above need a launch each (13 launches of 2-8 us for a
 // few thousand rows; one request of N = 2,000, rank 20, spent 115 us an iteration,
-// 7 of them in its MVM).  The vectors are in shared memory; element-wise steps
+// 7 of them in its MVM).  tail_ok says up to which sizes.  The vectors are in shared memory; element-wise steps
 // take element tid + 1024 m, the dots and Gram sums thread t of a 256-thread group
 // elements 2048 ch + 256 q + t of chunk ch, as in dots_kernel's and gram_kernel's blocks.
 // Every sum runs in the order of the kernels it stands for, so the results are the
 // same bit for bit: the split sums of the MVM, the float-float dots, the Gram
-// coefficients, the Woodbury apply (32-row blocks, FP64 across them).
+// coefficients, the Woodbury apply (32-row blocks, FP64 across them; wb_ltw_kernel takes
+// larger blocks above 64 rows per SM, so there, on fewer than 128 SMs, L^T r differs by
+// rounding).
 constexpr int kTailMaxN = 4 * kDotChunk;
 constexpr int kTailThreads = 1024;
 struct TailParams {
@@ -916,19 +918,33 @@ int CgSolver::start(bool from_x, int k0) {
     return flag_copy();
 }
 
-// The one-launch rest of an iteration: up to kTailMaxN rows, and as long as one CTA
-// reads its column's share (the factor twice, the bases) faster than thirteen launches
-// start: see the figures at cg_tail_kernel.
-bool CgSolver::tail_ok() const { return N <= kTailMaxN && N * (int64_t)(rank + 32) <= 600000; }
+// Whether the rest of this iteration runs as one launch: up to kTailMaxN rows, and while the
+// launches it saves (36 us; 16 more for the Woodbury apply) are worth more than what one CTA
+// per column loses on reading the factor and the nb stored bases through one SM. Per column of
+// the factor and per basis vector and pass, that loss was fitted to both paths' times (one
+// column of the right-hand side unless R is given; us a step, general / one launch):
+//   N = 2,000: rank 20 104 / 50, rank 200 124 / 113; 250 bases 138 / 80
+//   N = 4,000: rank 20 110 / 65, rank 100 118 / 111, rank 200 128 / 160; 350 bases 183 / 173
+//   N = 6,000: rank 20 119 / 87, rank 60 125 / 121, rank 100 127 / 155; 76 bases 118 / 114, 126 125 / 149
+//   N = 8,000: rank 20 133 / 108, rank 60 138 / 147; 76 bases 136 / 134, 350 199 / 326;
+//              R = 17, 126 bases 226 / 345; R = 64, 38 bases 194 / 190, 126 bases 282 / 361
+// (up to 2,048 rows four groups of warps share the bases, up to 4,096 two, beyond that none).
+bool CgSolver::tail_ok(int nb) const {
+    if (N > kTailMaxN) return false;
+    const double n = 1e-3 * (double)N;
+    const double per_rank = 0.1 + 0.06 * n + 0.0065 * n * n;
+    const double per_basis = N <= kDotChunk ? 0.0 : N <= 2 * kDotChunk ? 0.1 : 0.45 + 0.013 * R;
+    return rank * per_rank + passes * nb * per_basis <= (rank > 0 ? 52.0 : 36.0);
+}
 
-int CgSolver::tail(const MvmParts& parts, KOp& mvm) {
+int CgSolver::tail(const MvmParts& parts, KOp& mvm, int nb) {
     TailParams p;
     const size_t NR = (size_t)N * R;
     p.N = (int)N;
     p.R = R;
     p.nblk = b.nblk_dot;
     p.k = k;
-    p.nb = k - nb0 + 1;   // basis vectors r_0 .. r_k of this run
+    p.nb = nb;
     p.passes = passes;
     p.reorth = reorth;
     p.stable = stable;
@@ -975,18 +991,19 @@ int CgSolver::iterate() {
     const size_t NR = (size_t)N * R;
     // Kd = Ktilde d
     KOp& mvm = escalated ? *op_chk : refined ? *op_ref : op;
-    if (tail_ok()) {
+    const int nb = k - nb0 + 1;   // basis vectors r_0 .. r_k of this run
+    if (tail_ok(reorth != GP_REORTH_NONE ? nb : 0)) {
         MvmParts parts;
         GPK_TRY(kop_apply(ctx, mvm, b.d, R, b.Kd, N, true, s, &parts, v_ready_op == &mvm));
-        return tail(parts, mvm);
+        return tail(parts, mvm, nb);
     }
+    v_ready_op = nullptr;   // the general path rewrites d alone
     GPK_TRY(kop_apply(ctx, mvm, b.d, R, b.Kd, N, true, s));
     GPK_TRY(dots(b.d, b.Kd, true));   // masked by the flags of the last scalar step
     GPK_TRY(scalar(SC_ALPHA, k));
     update_xr_kernel<<<gcol, 256, 0, s>>>(U, b.r, b.d, b.Kd, N, b.st);
     GPK_TRY(launched(1));
     if (reorth != GP_REORTH_NONE) {
-        const int nb = k - nb0 + 1;   // basis vectors r_0 .. r_k of this run
         const float* ZB = reorth == GP_REORTH_PINV ? b.zeta : b.rho;
         for (int p = 0; p < passes; ++p) {
             gram_kernel<<<gdot, kDotThreads, (size_t)(kDotThreads / 32) * nb * sizeof(float), s>>>(
@@ -1000,7 +1017,7 @@ int CgSolver::iterate() {
     GPK_TRY(precond(b.r, b.z, true));
     GPK_TRY(dots(b.r, b.z, true));
     GPK_TRY(scalar(SC_BETA, k));
-    const size_t slot = (size_t)(k - nb0 + 1);
+    const size_t slot = (size_t)nb;
     float* rho_k = b.rho ? b.rho + slot * NR : nullptr;
     float* zeta_k = b.zeta ? b.zeta + slot * NR : nullptr;
     update_d_kernel<<<gcol, 256, 0, s>>>(b.d, b.z, b.r, N, b.st, 0, reorth, rho_k, zeta_k);
@@ -1068,7 +1085,7 @@ int CgSolver::setup(Ctx* c, WsCarver& wc, const gp_hyp_t* h, const float* X_, in
         }
     }
     wc_rest = wc;
-    if (tail_ok())
+    if (N <= kTailMaxN)
         GPK_CUDA_TRY(cudaFuncSetAttribute(cg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)tail_smem(kTailMaxN)));
     vg = vec_grid(ctx, N);

@@ -328,8 +328,8 @@ struct CgSolver {
     int finish(gp_cg_stats_t* stats);        // blocking: copy back, summarize
 
   private:
-    bool tail_ok() const;
-    int tail(const MvmParts& parts, KOp& mvm);
+    bool tail_ok(int nb) const;   // nb: stored basis vectors
+    int tail(const MvmParts& parts, KOp& mvm, int nb);
     const KOp* v_ready_op = nullptr;   // operator whose FP32 copy of d the last tail kernel wrote
     int launched(int n);
     int flag_copy();

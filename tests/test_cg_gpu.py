@@ -399,3 +399,79 @@ def test_one_launch_iteration_matches_general_path(ctx, alg, reorth, passes, pre
         out.append((U.cpu().numpy()[:, -8192:].astype(np.float64), info["alpha"][:6], info["beta"][:5]))
     for a, b in zip(*out):
         assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
+
+
+def _padded(pc, rank):
+    """The same preconditioner with columns of zeros appended to L (and 1 on the diagonal of the
+    core): the same sums with zeros added, and a rank that the one-launch iteration leaves to
+    the general path."""
+    from paper_2207_06856_gb300 import gpk
+    N, k = pc.L.shape[1], pc.rank
+    L = torch.zeros((rank, N), dtype=torch.float32, device="cuda:0")
+    L[:k] = pc.L
+    core = torch.eye(rank, dtype=torch.float64, device="cuda:0")
+    core[:k, :k] = pc.core
+    return gpk.Precond(L, core, pc.piv, rank)
+
+
+def _tail_problem(N, R, seed):
+    """A slowly converging system (Matern-1/2 in 3 dimensions, noise 1e-3): hundreds of steps."""
+    from paper_2207_06856_gb300 import gpk
+    r = np.random.default_rng(seed)
+    X, V = r.standard_normal((N, 3)).astype(np.float32), r.standard_normal((R, N)).astype(np.float32)
+    return gpk.Hyper(2, np.ones(3, np.float32), 1.0, 1e-3), _dev(X), _dev(V)
+
+
+def _tail_flags(prec):
+    from paper_2207_06856_gb300 import gpk
+    return {"fp32": gpk.FP32, "fp16": gpk.FP16, "bf16": gpk.BF16, "hilo": gpk.FP16 | gpk.MVM_PSPLIT | gpk.MVM_XSPLIT,
+            "fp32_pv": gpk.FP16 | gpk.MVM_XSPLIT | gpk.MVM_FP32_PV}[prec]
+
+
+# one to four dot chunks of 2,048 rows, and their edges; the last two cross over to the general
+# path on the way, at N = 8,000 near 70 bases
+TAIL_BITS = [(300, 4, "fp32_pv", 20, "pinv", 1, 12), (700, 1, "fp32", 20, "pinv", 1, 12),
+             (2048, 3, "hilo", 31, "pinv", 2, 12), (2049, 1, "fp32_pv", 20, "pinv", 1, 12),
+             (2500, 17, "fp16", 1, "euclid", 2, 12), (4096, 5, "bf16", 20, "pinv", 1, 12),
+             (5000, 2, "fp32_pv", 33, "none", 1, 12), (8191, 33, "hilo", 7, "pinv", 1, 12),
+             (8192, 2, "hilo", 20, "pinv", 1, 40), (8000, 2, "fp32_pv", 20, "pinv", 1, 130),
+             (6001, 3, "hilo", 20, "pinv", 2, 100)]
+
+
+@pytest.mark.parametrize("N,R,prec,rank,reorth,passes,iters", TAIL_BITS)
+def test_one_launch_iteration_bit_identical(ctx, N, R, prec, rank, reorth, passes, iters):
+    """One launch after each MVM (its own sum of the MVM's partial results, its own FP32 copy of
+    the next direction) against the general path on the same system, bit for bit."""
+    from paper_2207_06856_gb300 import gpk
+    if torch.cuda.get_device_properties(0).multi_processor_count < 128:
+        pytest.skip("the Woodbury apply sums other blocks of rows on fewer than 128 SMs")
+    hyp, X, V = _tail_problem(N, R, N + R)
+    pc = gpk.pivchol_precond(ctx, hyp, X, rank)
+    out = []
+    for p in (pc, _padded(pc, 512)):
+        n0 = ctx.launches
+        U, _, info = gpk.cg_solve(ctx, hyp, X, V, p, tol=0.0, min_iter=iters, max_iter=iters, restarts=0, reorth=reorth,
+                                  reorth_passes=passes, precision=_tail_flags(prec), escalate=False)
+        ctx.check()
+        out.append((ctx.launches - n0, U.cpu().numpy(), info["alpha"], info["beta"][:-1], info["resid_hist"]))
+    assert out[1][0] - out[0][0] >= 8 * min(iters, 30)   # they did take different paths
+    for a, b in zip(out[0][1:], out[1][1:]):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,R,passes", [(8000, 1, 1), (8000, 17, 1), (6000, 17, 2)])
+def test_one_launch_iteration_ends_with_many_bases(ctx, N, R, passes):
+    """One CTA per column reads all stored bases: beyond some number of them the general path,
+    which spreads that read over the GPU, is the faster one and is taken. Steps are counted by
+    their launches, 8 or more fewer on the one-launch path."""
+    from paper_2207_06856_gb300 import gpk
+    hyp, X, V = _tail_problem(N, R, 3)
+    pc = gpk.pivchol_precond(ctx, hyp, X, 20)
+    n = []
+    for iters in (1, 11, 150, 160):
+        n0 = ctx.launches
+        gpk.cg_solve(ctx, hyp, X, V, pc, tol=0.0, min_iter=iters, max_iter=iters, restarts=0, reorth_passes=passes,
+                     precision=_tail_flags("fp32_pv" if R == 1 else "hilo"), escalate=False)
+        ctx.check()
+        n.append(ctx.launches - n0)
+    assert n[3] - n[2] >= (n[1] - n[0]) + 10 * 8
