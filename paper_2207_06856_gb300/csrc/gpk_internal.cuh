@@ -231,6 +231,14 @@ int kop_prepare(Ctx* ctx, WsCarver& wc, KOp& op, const gp_hyp_t* hyp, const floa
 int kop_apply(Ctx* ctx, KOp& op, const float* V, int R, float* out, int64_t ld_out, bool add_noise, cudaStream_t s,
               MvmParts* parts = nullptr, bool v_ready = false);
 
+// Dynamic shared memory a kernel may be launched with.  The limit belongs to the function, not to
+// the launch: `bytes` is the kernel's maximum, the same at every call, so that a thread that
+// launches it with little never lowers the limit under another thread's launch with more.
+template <class F>
+inline cudaError_t allow_smem(F* fn, size_t bytes) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // Tensor-map helper (driver entry point fetched through the runtime).
 int encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uint64_t inner, uint64_t outer,
                    uint64_t row_bytes, uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz);

@@ -466,7 +466,7 @@ cudaError_t launch_tc_typed(const TcPlan& plan, const TcParams& prm, const CUten
                             const CUtensorMap& v, cudaStream_t s) {
     const int smem = tc_smem_bytes(plan.k_pad, plan.R_pad, prm.vsplit);
     auto kfn = kmvm_tc_kernel<KIND, BF16, PSPLIT>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kfn, kMaxSmemBytes - 512);   // (the sizes tc_stages accepts are multiples of 4 KB plus 1)
     if (e != cudaSuccess) return e;
     kfn<<<plan.grid, kThreads, smem, s>>>(a, b, v, prm);
     return cudaGetLastError();

@@ -796,7 +796,7 @@ cudaError_t launch_tp_mode(const TcPlan& plan, const TpParams& prm, const CUtens
                            const CUtensorMap& v, cudaStream_t s) {
     const TpSmem& m = prm.sm;
     auto kfn = kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV, MODE, NG>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.total);
+    cudaError_t e = allow_smem(kfn, kMaxSmemBytes - 512);
     if (e != cudaSuccess) return e;
     kfn<<<plan.grid, tp_threads(MODE), m.total, s>>>(a, b, v, prm);
     return cudaGetLastError();

@@ -518,7 +518,8 @@ size_t pivchol_workspace(const Ctx* ctx, int64_t N, int d, int rank) {
 
 namespace {
 // Shared memory of the one-CTA core kernels: a vector, and the k x k matrix when it fits 200 KB (k <= 159).
-int core_in_smem(int k) { return (size_t)(k + 1) * k * sizeof(double) <= 200 * 1024 ? 1 : 0; }
+constexpr size_t kCoreSmem = 200 * 1024;
+int core_in_smem(int k) { return (size_t)(k + 1) * k * sizeof(double) <= kCoreSmem ? 1 : 0; }
 size_t core_smem(int k) { return (size_t)(core_in_smem(k) ? (k + 1) * k : k) * sizeof(double); }
 }  // namespace
 
@@ -585,9 +586,7 @@ int pivchol_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int
     core_sum_kernel<<<(kr * kr + 127) / 128, 128, 0, s>>>(part, nsplit, kr, 1.0 / hyp->noise, core);
     const int in_smem = core_in_smem(kr);
     const size_t sh = core_smem(kr);
-    if (sh > 48 * 1024 && cudaFuncSetAttribute(core_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) !=
-                              cudaSuccess)
-        return GP_ERR_CUDA;
+    if (allow_smem(core_chol_kernel, kCoreSmem) != cudaSuccess) return GP_ERR_CUDA;
     core_chol_kernel<<<1, 512, sh, s>>>(kr, in_smem, core, ctx->dev_err);
     ctx->launches += 3;
     return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
@@ -624,9 +623,7 @@ int woodbury_prepare(Ctx* ctx, const double* core, int k, double* cinv, cudaStre
     const int in_smem = core_in_smem(k);
     const size_t sh = core_smem(k);
     auto fn = k <= 128 ? core_inverse_kernel<4> : (k <= 256 ? core_inverse_kernel<8> : core_inverse_kernel<16>);
-    if (sh > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) != cudaSuccess)
-        return GP_ERR_CUDA;
+    if (allow_smem(fn, kCoreSmem) != cudaSuccess) return GP_ERR_CUDA;
     fn<<<g, 128, sh, s>>>(core, k, in_smem, cinv);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;

@@ -786,7 +786,7 @@ int vjp_tc_run(Ctx* ctx, WsCarver& wc, const gp_hyp_t* hyp, const float* X, int6
 #define GPK_VJP_CASE(K)                                                                                   \
     case K: {                                                                                             \
         auto fn = kvjp_tc_kernel<K>;                                                                      \
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.total);          \
+        e = allow_smem(fn, kMaxSmemBytes - 512);                                                          \
         if (e == cudaSuccess) {                                                                           \
             fn<<<pl.grid, kThreads, m.total, s>>>(op.tmA, op.tmB, tmUW, tmWU, tmXt, prm);                  \
             e = cudaGetLastError();                                                                       \
