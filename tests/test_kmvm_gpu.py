@@ -560,3 +560,15 @@ def test_skip_tiles_runs_of_empty_items(ctx, R, flags_name, square):
     ev, tot = gpk.kmvm_tile_count(ctx, gpk.Hyper(0, ls, 1.0, 0.05), torch.from_numpy(X).to(dev),
                                   None if square else torch.from_numpy(Xc).to(dev), flags=base | gpk.MVM_SKIP_TILES)
     assert 0 < ev < 0.15 * tot, (ev, tot)
+
+
+@pytest.mark.parametrize("d,R", [(9, 1), (12, 4), (13, 2), (16, 3), (16, 4), (17, 4), (8, 4), (16, 5)])
+@pytest.mark.parametrize("N", [1, 63, 65, 66, 67, 257])
+def test_fp32_column_loop_edges(ctx, N, d, R):
+    """The FP32 engine's two column loops (9 to 16 dimensions with up to 4 vectors, and the
+    others) where the last tile of 64 columns leaves 1 to 3 of them over. Each output against
+    the FP32 tolerance times the sum of its terms' magnitudes."""
+    for kern in range(4):
+        X, V, _, ls, a2, s2 = workloads.random_problem(N, d, R, seed=N + d + kern, kernel=kern)
+        got = _run(ctx, X, V, kern, ls, a2, s2, "fp32")
+        assert np.all(np.abs(got - _ref(X, V, kern, ls, a2, s2)) <= TOL["fp32"] * _ref(X, np.abs(V), kern, ls, a2, s2))
