@@ -126,7 +126,8 @@ struct TpBarriers {
     uint64_t empty[kMaxStages];
     // S and P buffers, [2 x ring slot + row tile]
     uint64_t s_full[kMaxBufs];
-    uint64_t p_empty[kMaxBufs]; // P consumed by its value product (and, in place, S may be rewritten)
+    uint64_t p_empty[kMaxBufs]; // P consumed by its value product (and, in place, S may be rewritten);
+                                // FP32 value product: S read by the row tile's epilogue warps
     uint64_t o_full[2];         // per row tile, once per item with an evaluated tile
     uint64_t xi_full[2];
     uint64_t xi_empty[2];
@@ -136,8 +137,8 @@ struct TpBarriers {
 // Named barriers between the 8 epilogue warps of a row tile (arrive) and its
 // issuer (sync): S read into registers, P stored.  id 0 is __syncthreads.
 constexpr uint32_t kBarThreads = 9 * 32;
-constexpr uint32_t bar_s_read(uint32_t buf) { return 1u + buf; }    // buf = 2 x ring slot + row tile < 4
-constexpr uint32_t bar_p_full(uint32_t buf) { return 5u + buf; }    // < 6
+constexpr uint32_t bar_s_read(uint32_t w) { return 1u + w; }        // WIDE: row tile
+constexpr uint32_t bar_p_full(uint32_t buf) { return 3u + buf; }    // 2 x ring slot + row tile < 6
 
 // WIDE (P beside S), in place (P over S, NG buffers per row tile), or FP32 value product.
 enum TpMode { kWide = 0, kInPlace = 1, kSpv = 2 };
@@ -400,24 +401,20 @@ __device__ void tp_issuer_s(const TpParams& p, TpBarriers& bars, const uint8_t* 
     if (!si.ok && (threadIdx.x & 31) == 0) record_error(p.err, DEV_TIMEOUT);
 }
 
-// Issuer of row tile w for the FP32 value product: S only, two buffers.
+// Issuer of row tile w for the FP32 value product: S only, two buffers, each refilled once the
+// row tile's epilogue warps have read it (p_empty, one arrival per warp). Here the waits are
+// mbarriers with the suspend-time hint on both sides: this epilogue is bound by issue slots and
+// registers, and one named barrier more in its loop spilled. N = 65,536, d = 8, hi + lo inputs, RBF, us
+// a call for 1, 2 and 4 columns: named barrier 795 / 1,203 / 2,171, this form 770 / 1,138 / 2,089.
 template <int NG>
 __device__ void tp_issuer_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
                               uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
     TpSIssue<kSpv, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
-    uint32_t n = 0;
-    for (si.next(); si.have; si.next(), ++n) {
-        if (n >= NG) ptx::bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
+    for (si.next(); si.have; si.next()) {
+        si.ok = si.ok &&
+                __all_sync(0xffffffffu, ptx::mbar_wait_sleep(&bars.p_empty[2u * si.b + w], si.bph, p.limit_ns));
         si.issue(0);
         si.next_stage();
-    }
-    for (uint32_t q = 0; q < (n < NG ? n : NG); ++q) {   // the epilogue's last reads
-        if (n >= NG) {
-            ptx::bar_sync(bar_s_read(2u * si.b + w), kBarThreads);
-            if (++si.b == NG) si.b = 0;
-        } else {
-            ptx::bar_sync(bar_s_read(2u * q + w), kBarThreads);
-        }
     }
     ptx::mma_commit_elect(&bars.drain[w]);
     warp_wait(&bars.drain[w], 0, p.limit_ns);
@@ -620,8 +617,8 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
 // with FP32 FMAs, v_j read in FP32 from the stage (TMA box of 128 columns x 4
 // rows; this warpgroup's 64 columns; broadcast 16-byte reads).  No P and no
 // value-product MMAs: no rounding of the kernel values, and
-// one column takes 0.763 ms against 0.835 on the hi + lo tile (N = 65,536, d = 8, RBF;
-// four columns 2.13 against 0.84).  Each warp releases
+// one column takes 770 us a call against 867 on the hi + lo tile (N = 65,536, d = 8, RBF;
+// two 1,137 and four 2,088, where the hi + lo tile's time hardly changes).  Each warp releases
 // the stage after its reads (16 arrivals), and writes its row sums of the item
 // to the partial rows ch * R + r, which the split reduction adds up.
 template <int KIND, int RN>
@@ -632,7 +629,7 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
     const int row = wq * 32 + lane;
     const uint32_t S = (uint32_t)p.stages;
     const uint32_t stage_bytes = xbytes + vtbytes;
-    uint32_t gt = 0, st = 0, ph = 0;
+    uint32_t g = 0, st = 0, ph = 0;   // evaluated tiles; stage ring slot and its fill parity
     bool ok = true;
 #pragma unroll 1
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
@@ -642,23 +639,27 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
         float acc[RN];
 #pragma unroll
         for (int r = 0; r < RN; ++r) acc[r] = 0.0f;
-        uint32_t t = 0;
 #pragma unroll 1
         for (int jt = j0; jt < j1; ++jt) {
             if (!tile_on(p, ip, jt)) continue;
-            const uint32_t g = gt + t, buf = g & 1u;
+            const uint32_t buf = g & 1u;
             // hinted waits: a spinning warp would take the issue slots of the warps computing
             // beside it and of the S issuer on its scheduler (this epilogue is issue-bound)
-            ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait_sleep(&bars.s_full[2 * buf + tl], (g >> 1) & 1, p.limit_ns) &&
-                                                   ptx::mbar_wait_sleep(&bars.full[st], ph, p.limit_ns));
+            if (!__all_sync(0xffffffffu, ptx::mbar_wait_sleep(&bars.s_full[2 * buf + tl], (g >> 1) & 1, p.limit_ns) &&
+                                             ptx::mbar_wait_sleep(&bars.full[st], ph, p.limit_ns))) {
+                ok = false;
+                break;
+            }
             ptx::tc_fence_after();
             const uint32_t tS = tmem + lane_off + buf * 256u + (uint32_t)tl * 128u + (uint32_t)ch * 64u;
             const bool dtile = (KIND == GP_KERNEL_MATERN12) && p.diag && (jt == it);
             const float* vb = reinterpret_cast<const float*>(sSt + st * stage_bytes + xbytes) + ch * 64;
             // one 32-column half of S at a time (the register budget of 608 threads); the
             // buffer is released after the second load, while S of the next tile is
-            // already being formed in the other one
-#pragma unroll
+            // already being formed in the other one. From two columns on the halves are a loop
+            // (two columns, as above: 1,169 us unrolled with 8 bytes of spills, 1,138 as a loop; one
+            // column, Matern-3/2: 1,608 unrolled, 1,881 as a loop)
+#pragma unroll(RN == 1 ? 2 : 1)
             for (int hh = 0; hh < 2; ++hh) {
                 uint32_t rr[32];
                 ptx::tmem_ld32(tS + 32u * (uint32_t)hh, rr);
@@ -666,7 +667,8 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
                 ptx::tmem_reg_fence(rr);
                 if (hh == 1) {
                     ptx::tc_fence_before();
-                    ptx::bar_arrive(bar_s_read(2u * buf + (uint32_t)tl), kBarThreads, ok);
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&bars.p_empty[2u * buf + (uint32_t)tl]);
                 }
 #pragma unroll
                 for (int c4 = 0; c4 < 4; ++c4) {      // 16-byte chunk c: columns [8 c, 8 c + 8) of the 64
@@ -701,14 +703,14 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&bars.empty[st]);   // this warp is done with the stage's Vt
             if (++st == S) { st = 0; ph ^= 1u; }
-            ++t;
+            ++g;
         }
+        if (!ok) break;
 #pragma unroll
         for (int r = 0; r < RN; ++r)   // RN = 1, 2 or 4 (3 runs as 4: the fourth row of v is zero)
             if (r < p.nrhs)
                 p.partial[((int64_t)(2 * sp + ch) * p.nrhs + r) * p.ld_part + (int64_t)ip * kPairRows + tl * kBM + row] =
                     acc[r];
-        gt += t;
     }
     if (!ok) record_error(p.err, DEV_TIMEOUT);
 }
@@ -737,7 +739,7 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
         for (int b = 0; b < kMaxBufs; ++b) {
             ptx::mbar_init(&bars.s_full[b], 1);
-            ptx::mbar_init(&bars.p_empty[b], 1);
+            ptx::mbar_init(&bars.p_empty[b], SPV ? kEpiWarps / 2 : 1);
         }
 #pragma unroll 1
         for (int b = 0; b < 2; ++b) {
