@@ -164,13 +164,47 @@ __device__ __forceinline__ void item_range(const TpParams& p, int item, int& ip,
     j1 = (int)((q + 1u) * (uint32_t)p.n_jt / (uint32_t)p.n_split);
 }
 
-// Whether the column tile jt of row-tile pair ip is evaluated (compact support:
-// a cleared bit means every kernel value of the pair rounds to zero).
-__device__ __forceinline__ bool tile_on(const TpParams& p, int ip, int jt) {
-    return !p.mask || ((__ldg(p.mask + (int64_t)ip * p.mask_words + (jt >> 5)) >> (jt & 31)) & 1u);
+// Tile skipping (SKIP; compact support): a cleared bit of the mask means every kernel value of
+// (row-tile pair ip, column tile jt) rounds to zero. Every role goes through the mask for itself, a
+// word of 32 tiles at a time; the issuers take the stages as they come and need the number of
+// tiles alone. Tile by tile, in one kernel for both cases: 0.260 ms a launch for 16 far-apart clusters
+// (N = 65,536, d = 8, 17 columns, 1 tile in 16 evaluated) and, for 64 clusters, d = 3, 336 us a call at
+// N = 65,536 and 992 at 131,072; like this 0.116 ms, 170 and 318 us.
+
+// Evaluated column tiles of pair ip in [j0, j1).
+template <int SKIP>
+__device__ __forceinline__ int tile_count(const TpParams& p, int ip, int j0, int j1) {
+    if constexpr (!SKIP) return j1 - j0;
+    const uint32_t* m = p.mask + (int64_t)ip * p.mask_words;
+    int n = 0;
+#pragma unroll 1
+    for (int w = j0 >> 5; 32 * w < j1; ++w) {
+        uint32_t bits = __ldg(m + w);
+        if (32 * w < j0) bits &= 0xffffffffu << (j0 - 32 * w);
+        if (32 * w + 32 > j1) bits &= 0xffffffffu >> (32 * w + 32 - j1);
+        n += __popc(bits);
+    }
+    return n;
+}
+// The first evaluated column tile of pair ip in [jt, j1), or j1.
+template <int SKIP>
+__device__ __forceinline__ int next_tile(const TpParams& p, int ip, int jt, int j1) {
+    if constexpr (!SKIP) return jt;
+    if (jt >= j1) return j1;
+    const uint32_t* m = p.mask + (int64_t)ip * p.mask_words;
+    int w = jt >> 5;
+    uint32_t bits = __ldg(m + w) & (0xffffffffu << (jt & 31));
+#pragma unroll 1
+    while (bits == 0u) {
+        if (32 * ++w >= j1) return j1;
+        bits = __ldg(m + w);
+    }
+    jt = 32 * w + __ffs((int)bits) - 1;
+    return jt < j1 ? jt : j1;
 }
 
 // ---- TMA producer (one thread) ------------------------------------------------
+template <int SKIP>
 __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUtensorMap* tmB,
                             const CUtensorMap* tmV, TpBarriers& bars, uint8_t* sSt, uint8_t* sXi, uint32_t xbytes,
                             uint32_t vtbytes) {
@@ -192,8 +226,7 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
         ptx::tma_load_2d(sX + xbytes, tmA, &bars.xi_full[xb], 0, ip * kPairRows + kBM);
         ++xi_loads;
 #pragma unroll 1
-        for (int jt = j0; jt < j1; ++jt) {
-            if (!tile_on(p, ip, jt)) continue;
+        for (int jt = next_tile<SKIP>(p, ip, j0, j1); jt < j1; jt = next_tile<SKIP>(p, ip, jt + 1, j1)) {
             const uint32_t st = fills % S, u = fills / S;
             if (u > 0 && !ptx::mbar_wait_sleep(&bars.empty[st], (u - 1) & 1, p.limit_ns)) { ok = false; break; }
             uint8_t* sx = sSt + st * (xbytes + vtbytes);
@@ -239,13 +272,14 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64
 
 // Walks the column tiles whose S is issued; runs one tile ahead of the value
 // product, across items.
-template <int MODE, int NG>
+template <int MODE, int NG, int SKIP>
 struct TpSIssue {
     using T = TpTmem<MODE, NG>;
     const TpParams& p;
     TpBarriers& bars;
     uint32_t aSt, aXi0, xbytes, stage_bytes, arow, hi_x, tmem, id, w, s_full;
-    int item, jt, j1, ip, xb;
+    int item, xb = 0;
+    int left = 0;               // evaluated tiles of the item still to be selected
     uint32_t ic = 0;            // items entered
     uint32_t st = 0, ph = 0;    // stage ring slot and its fill parity
     uint32_t b = 0, bph = 1;    // buffer ring slot; parity of its last release (first round: passes at once)
@@ -261,26 +295,22 @@ struct TpSIssue {
         hi_x = ptx::smem_desc_hi(8u * arow, (arow == 32) ? 6u : (arow == 64 ? 4u : 2u));
         s_full = ptx::smem_u32(&bars.s_full[w]);
         item = (int)blockIdx.x - (int)gridDim.x;
-        jt = j1 = 0;
     }
     // Select the next evaluated tile; have = false after the last.
     __device__ __forceinline__ void next() {
-        ++jt;
 #pragma unroll 1
         while (have) {
-            if (jt < j1) {
-                if (tile_on(p, ip, jt)) {
-                    ok = ok && warp_wait(&bars.full[st], ph, p.limit_ns);
-                    return;
-                }
-                ++jt;
-                continue;
+            if (left > 0) {
+                --left;
+                ok = ok && warp_wait(&bars.full[st], ph, p.limit_ns);
+                return;
             }
             if (ic > 0 && ok) ptx::mma_commit_elect(&bars.xi_empty[xb]);   // the row tile's last use in its item
             item += (int)gridDim.x;
             if (item >= p.n_items) { have = false; return; }
-            int sp;
-            item_range(p, item, ip, sp, jt, j1);
+            int ip, sp, j0, j1;
+            item_range(p, item, ip, sp, j0, j1);
+            left = tile_count<SKIP>(p, ip, j0, j1);
             xb = p.xi_bufs == 2 ? (int)(ic & 1u) : 0;
             ok = ok && warp_wait(&bars.xi_full[xb], (p.xi_bufs == 2 ? ic >> 1 : ic) & 1u, p.limit_ns);
             ++ic;
@@ -325,11 +355,11 @@ __device__ __forceinline__ void tp_value_product(uint32_t tO, uint32_t tP, uint3
 // WIDE, issuer of row tile w: S(t + 1) once the epilogue holds S(t) in registers,
 // then O += P(t) Vt^T once it has stored P(t).  In place, value-product issuer
 // (the S issuer of tp_issuer_s refills the buffers): O += P(q) Vt^T for each slot.
-template <int MODE, int NG, int PSPLIT>
+template <int MODE, int NG, int PSPLIT, int SKIP>
 __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi, uint32_t xbytes,
                           uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t id_pv, uint32_t w) {
     using T = TpTmem<MODE, NG>;
-    TpSIssue<MODE, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+    TpSIssue<MODE, NG, SKIP> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
     const uint32_t lV0 = ptx::smem_desc_lo(ptx::smem_u32(sSt) + xbytes), kb = (uint32_t)p.rv * 8u;
     const uint32_t p_empty = ptx::smem_u32(&bars.p_empty[w]);
     const uint32_t tO = tmem + T::o(w);
@@ -345,8 +375,7 @@ __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sS
         uint32_t acc = 0;   // 0 for the item's first product (the epilogue has read O of the last item before
                             // it stores this item's first P)
 #pragma unroll 1
-        for (int jt = j0; jt < j1; ++jt) {
-            if (!tile_on(p, ip, jt)) continue;
+        for (int n = tile_count<SKIP>(p, ip, j0, j1); n > 0; --n) {
             const uint32_t lV = lV0 + st * (stage_bytes >> 4);
             if constexpr (MODE == kWide) {
                 // (this tile's stage landed before its S was issued)
@@ -383,10 +412,10 @@ __device__ void tp_issuer(const TpParams& p, TpBarriers& bars, const uint8_t* sS
 
 // In place, S issuer of row tile w: S of each slot (64 columns of a tile) once the
 // value product of the slot NG before it in the ring has completed.
-template <int NG>
+template <int NG, int SKIP>
 __device__ void tp_issuer_s(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
                             uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
-    TpSIssue<kInPlace, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+    TpSIssue<kInPlace, NG, SKIP> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
 #pragma unroll 1
     for (si.next(); si.have && si.ok; si.next()) {
 #pragma unroll
@@ -406,10 +435,10 @@ __device__ void tp_issuer_s(const TpParams& p, TpBarriers& bars, const uint8_t* 
 // mbarriers with the suspend-time hint on both sides: this epilogue is bound by issue slots and
 // registers, and one named barrier more in its loop spilled. N = 65,536, d = 8, hi + lo inputs, RBF, us
 // a call for 1, 2 and 4 columns: named barrier 795 / 1,203 / 2,171, this form 770 / 1,138 / 2,089.
-template <int NG>
+template <int NG, int SKIP>
 __device__ void tp_issuer_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
                               uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
-    TpSIssue<kSpv, NG> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
+    TpSIssue<kSpv, NG, SKIP> si(p, bars, sSt, sXi, xbytes, stage_bytes, tmem, id_s, w);
     for (si.next(); si.have; si.next()) {
         si.ok = si.ok &&
                 __all_sync(0xffffffffu, ptx::mbar_wait_sleep(&bars.p_empty[2u * si.b + w], si.bph, p.limit_ns));
@@ -476,7 +505,7 @@ __device__ __forceinline__ void tp_values(const uint32_t (&r)[32], int col0, int
     }
 }
 
-template <int KIND, int BF16, int PSPLIT, int HS, int MODE, int NG>
+template <int KIND, int BF16, int PSPLIT, int HS, int MODE, int NG, int SKIP>
 __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, int wg, int wq, int lane) {
     using T = TpTmem<MODE, NG>;
     constexpr int H = kBN / (int)T::kS;
@@ -491,10 +520,9 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
         const int it = 2 * ip + tl;   // this warpgroup's row tile
-        bool any = false;             // a tile of this item was evaluated
+        const bool any = !SKIP || next_tile<SKIP>(p, ip, j0, j1) < j1;
 #pragma unroll 1
-        for (int jt = j0; jt < j1; ++jt) {
-            if (!tile_on(p, ip, jt)) continue;
+        for (int jt = next_tile<SKIP>(p, ip, j0, j1); jt < j1; jt = next_tile<SKIP>(p, ip, jt + 1, j1)) {
             const bool dtile = (KIND == GP_KERNEL_MATERN12) && p.diag && (jt == it);
 #pragma unroll
             for (int h = 0; h < H; ++h) {
@@ -564,7 +592,6 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
                 ptx::bar_arrive(bar_p_full(buf), kBarThreads, ok);
                 if (++b == NG) { b = 0; ph ^= 1u; }
             }
-            any = true;
         }
         // O read-out: lanes are rows of the tile; this warpgroup's half of the right-hand sides.
         if (any) {
@@ -621,7 +648,7 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
 // two 1,137 and four 2,088, where the hi + lo tile's time hardly changes).  Each warp releases
 // the stage after its reads (16 arrivals), and writes its row sums of the item
 // to the partial rows ch * R + r, which the split reduction adds up.
-template <int KIND, int RN>
+template <int KIND, int RN, int SKIP>
 __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, uint32_t xbytes,
                                 uint32_t vtbytes, uint32_t tmem, int wg, int wq, int lane) {
     const int tl = wg & 1, ch = wg >> 1;
@@ -640,8 +667,8 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
 #pragma unroll
         for (int r = 0; r < RN; ++r) acc[r] = 0.0f;
 #pragma unroll 1
-        for (int jt = j0; jt < j1; ++jt) {
-            if (!tile_on(p, ip, jt)) continue;
+        for (int n = tile_count<SKIP>(p, ip, j0, j1), jt = j0 - 1; n > 0; --n) {
+            if constexpr (KIND == GP_KERNEL_MATERN12) jt = next_tile<SKIP>(p, ip, jt + 1, j1);   // (the diagonal)
             const uint32_t buf = g & 1u;
             // hinted waits: a spinning warp would take the issue slots of the warps computing
             // beside it and of the S issuer on its scheduler (this epilogue is issue-bound)
@@ -716,7 +743,7 @@ __device__ void tp_epilogue_spv(const TpParams& p, TpBarriers& bars, const uint8
 }
 
 // MODE and NG as in TpTmem (in place: NG = 3 when O takes 64 columns per row tile, 2 when it takes 128).
-template <int KIND, int BF16, int PSPLIT, int HS, int SPV, int MODE, int NG>
+template <int KIND, int BF16, int PSPLIT, int HS, int SPV, int MODE, int NG, int SKIP>
 __global__ void __launch_bounds__(tp_threads(MODE), 1)
 kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmV, const TpParams p) {
@@ -763,7 +790,7 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tmem = tmem_slot;
 
     if (warp == kTmaWarp) {
-        if (lane == 0) tp_producer(p, &tmA, &tmB, &tmV, bars, sSt, sXi, m.xbytes, m.stage_bytes - m.xbytes);
+        if (lane == 0) tp_producer<SKIP>(p, &tmA, &tmB, &tmV, bars, sSt, sXi, m.xbytes, m.stage_bytes - m.xbytes);
         __syncwarp();
     } else if (warp >= kMmaWarp) {
         constexpr int kW = (int)TpTmem<MODE, NG>::kS;
@@ -771,21 +798,21 @@ kmvm_tp_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t w = (uint32_t)(warp - kMmaWarp) & 1u;
         if constexpr (MODE == kInPlace) {
             if (warp < kMmaWarp + 2)
-                tp_issuer_s<NG>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
+                tp_issuer_s<NG, SKIP>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
             else
-                tp_issuer<MODE, NG, PSPLIT>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
-                                            ptx::idesc_f16(kBM, p.rv, BF16), w);
+                tp_issuer<MODE, NG, PSPLIT, SKIP>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
+                                                  ptx::idesc_f16(kBM, p.rv, BF16), w);
         } else if constexpr (SPV > 0)
-            tp_issuer_spv<NG>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
+            tp_issuer_spv<NG, SKIP>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s, w);
         else
-            tp_issuer<MODE, NG, PSPLIT>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
-                                        ptx::idesc_f16(kBM, p.rv, BF16), w);
+            tp_issuer<MODE, NG, PSPLIT, SKIP>(p, bars, sSt, sXi, m.xbytes, m.stage_bytes, tmem, id_s,
+                                              ptx::idesc_f16(kBM, p.rv, BF16), w);
     } else {
         if constexpr (SPV > 0)
-            tp_epilogue_spv<KIND, SPV>(p, bars, sSt, m.xbytes, m.stage_bytes - m.xbytes, tmem, warp >> 2, warp & 3,
-                                       lane);
+            tp_epilogue_spv<KIND, SPV, SKIP>(p, bars, sSt, m.xbytes, m.stage_bytes - m.xbytes, tmem, warp >> 2,
+                                             warp & 3, lane);
         else
-            tp_epilogue<KIND, BF16, PSPLIT, HS, MODE, NG>(p, bars, tmem, warp >> 2, warp & 3, lane);
+            tp_epilogue<KIND, BF16, PSPLIT, HS, MODE, NG, SKIP>(p, bars, tmem, warp >> 2, warp & 3, lane);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -797,7 +824,8 @@ template <int KIND, int BF16, int PSPLIT, int HS, int SPV, int MODE, int NG>
 cudaError_t launch_tp_mode(const TcPlan& plan, const TpParams& prm, const CUtensorMap& a, const CUtensorMap& b,
                            const CUtensorMap& v, cudaStream_t s) {
     const TpSmem& m = prm.sm;
-    auto kfn = kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV, MODE, NG>;
+    auto kfn = prm.mask ? kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV, MODE, NG, 1>
+                        : kmvm_tp_kernel<KIND, BF16, PSPLIT, HS, SPV, MODE, NG, 0>;
     cudaError_t e = allow_smem(kfn, kMaxSmemBytes - 512);
     if (e != cudaSuccess) return e;
     kfn<<<plan.grid, tp_threads(MODE), m.total, s>>>(a, b, v, prm);

@@ -572,3 +572,24 @@ def test_fp32_column_loop_edges(ctx, N, d, R):
         X, V, _, ls, a2, s2 = workloads.random_problem(N, d, R, seed=N + d + kern, kernel=kern)
         got = _run(ctx, X, V, kern, ls, a2, s2, "fp32")
         assert np.all(np.abs(got - _ref(X, V, kern, ls, a2, s2)) <= TOL["fp32"] * _ref(X, np.abs(V), kern, ls, a2, s2))
+
+
+@pytest.mark.parametrize("mode,kern", [("fp16", 2), ("bf16", 2), ("fp32_pv", 0), ("fp32_pv", 2)])
+@pytest.mark.parametrize("N", [4000, 8191, 17000])
+def test_skip_tiles_walks_of_every_role(ctx, mode, kern, N):
+    """The roles walk the mask (the producer, and the Matern-1/2 epilogue for its diagonal) or count
+    its bits (the others), over column ranges that start and end anywhere in its 32-tile words:
+    the result stays bit-identical, or, with the kernel values in FP32, within the largest value
+    that counts as zero (2^-25) per term. Clusters 70 lengthscales apart, for Matern-1/2's tail."""
+    from paper_2207_06856_gb300 import gpk
+    g = (np.arange(4) - 1.5) * 70.0
+    X = _clusters(N // 16 + 1, [np.array([a, b, 0.0]) for a in g for b in g], 0.05, seed=N)[:N]
+    V = np.random.default_rng(N + 1).standard_normal((3, N)).astype(np.float32)
+    prec, fl = {"fp16": ("fp16", 0), "bf16": ("bf16", 0), "fp32_pv": ("fp16", gpk.MVM_FP32_PV)}[mode]
+    ls = np.ones(3, np.float32)
+    a = _run(ctx, X, V, kern, ls, 1.0, 0.05, prec, flags=fl)
+    b = _run(ctx, X, V, kern, ls, 1.0, 0.05, prec, flags=fl | gpk.MVM_SKIP_TILES)
+    assert np.array_equal(a, b) if mode != "fp32_pv" else np.allclose(a, b, rtol=0, atol=2.0 ** -24 * np.abs(V).sum())
+    ev, tot = gpk.kmvm_tile_count(ctx, gpk.Hyper(kern, ls, 1.0, 0.05), torch.from_numpy(X).to("cuda:0"), precision=prec,
+                                  flags=fl | gpk.MVM_SKIP_TILES)
+    assert ev < tot, (ev, tot)
