@@ -11,9 +11,12 @@
 // global argmax pass is needed; the kernel row is evaluated on the fly from
 // the scaled inputs (SIMT FP32, same kernel forms as the MVM).  A step is a chain
 // of latencies (launch, candidates, pivot row, the earlier columns, argmax), so
-// the launches overlap (programmatic dependent launch) and the earlier columns are
-// loaded sixteen at a time (the whole factor and core at N = 65,536, d = 8, rank 100:
-// 1.51 -> 0.95 ms a call; the core's 530 us and the inverse's 254 us are what the lines
+// a step is launched as a programmatic dependent of the one before (no step signals early: what
+// overlaps is the launch itself with the end of the last step) and the earlier columns are
+// loaded eight at a time (sixteen, with more registers, took longer at every size: N = 100,000,
+// d = 18, rank 100 1,428 against 1,324 us a call, rank 512 56.8 against 48.0 ms, where four at a
+// time had taken 55.5).  The whole factor and core at N = 65,536, d = 8, rank 100:
+// 1.51 -> 0.90 ms a call (the core's 530 us and the inverse's 254 us are what the lines
 // below took away).
 //
 // Core.  C = I + sigma^-2 L^T L is accumulated in FP64 from FP32 sums of
@@ -23,8 +26,8 @@
 // square roots and divisions off its chain (one reciprocal per column).
 //
 // Apply.  P^{-1} w = sigma^-2 w - sigma^-4 L C^{-1} L^T w: t = L^T w (FP32
-// within 256-row blocks, FP64 across blocks, fixed order), u = C^{-1} t by
-// FP64 triangular solves (one warp per right-hand side), then the N x k
+// within a block's rows, FP64 across blocks, fixed order), u = C^{-1} t with the
+// inverse formed once per solve (FP64, one warp per entry), then the N x k
 // product with u fused with the scaling.
 #include "gpk_internal.cuh"
 #include "kfun.cuh"
@@ -82,7 +85,7 @@ pivchol_step_kernel(const float* __restrict__ Xs, int64_t N, int dp, int m, floa
                     Cand* __restrict__ cout, int* __restrict__ piv, int* __restrict__ rank_out) {
     __shared__ __align__(16) float sxp[64];
     __shared__ float slp[512];
-    // launched while the previous step runs (programmatic dependent launch)
+    // programmatic dependent launch: the previous step's results are complete after this wait
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (*rank_out >= 0) return;   // an earlier step stopped the factorisation
     float dmax;
@@ -129,12 +132,12 @@ pivchol_step_kernel(const float* __restrict__ Xs, int64_t N, int dp, int m, floa
         float dot = 0.0f;
         const float* li = L + i;
         int q = 0;
-        for (; q + 16 <= m; q += 16) {   // sixteen loads in flight, the same order of additions
-            float v[16];
+        for (; q + 8 <= m; q += 8) {   // eight loads in flight, the same order of additions
+            float v[8];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = li[(int64_t)(q + u) * N];
+            for (int u = 0; u < 8; ++u) v[u] = li[(int64_t)(q + u) * N];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) dot = fmaf(v[u], slp[q + u], dot);
+            for (int u = 0; u < 8; ++u) dot = fmaf(v[u], slp[q + u], dot);
         }
 #pragma unroll 4
         for (; q < m; ++q) dot = fmaf(li[(int64_t)q * N], slp[q], dot);
