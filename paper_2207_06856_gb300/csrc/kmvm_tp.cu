@@ -76,7 +76,7 @@ constexpr uint32_t kSpvVBytes = 128u * 4u * 4u;   // FP32 value product: 128 col
 
 struct TpSmem {
     uint32_t xbytes, stage_bytes;
-    int stages, xi_bufs;
+    int stages;
     uint32_t total;   // dynamic shared memory to request (includes 1 KB alignment slack)
 };
 
@@ -87,8 +87,7 @@ __host__ __device__ inline TpSmem tp_smem(int k_pad, int rv) {
     m.xbytes = (uint32_t)kBM * (uint32_t)k_pad * 2u;
     m.stage_bytes = m.xbytes + 2u * (uint32_t)rv * 128u;
     m.stages = 0;
-    m.xi_bufs = 2;
-    const uint32_t fixed = 1024u + 4u * m.xbytes;
+    const uint32_t fixed = 1024u + 4u * m.xbytes;   // two buffers of the pair's row operands
     for (int s = kMaxStages; s >= 2; --s)
         if (fixed + (uint32_t)s * m.stage_bytes <= (uint32_t)kMaxSmemBytes - 512u) { m.stages = s; break; }
     m.total = fixed + (uint32_t)m.stages * m.stage_bytes;
@@ -102,7 +101,7 @@ struct TpParams {
     int n_ip, n_jt, n_split, n_items;
     int k_pad, rv;        // rv: rows of Vt per tile (N of the value product)
     int lo_off;           // row of Vt (column of O) where the lo parts start; 0: no lo parts
-    int stages, xi_bufs;
+    int stages;
     TpSmem sm;
     int nrhs;             // right-hand sides in use
     int spv;              // 1: FP32 value product; the V map is FP32, 128 columns x 4 rows per box
@@ -166,10 +165,11 @@ __device__ __forceinline__ void item_range(const TpParams& p, int item, int& ip,
 
 // Tile skipping (SKIP; compact support): a cleared bit of the mask means every kernel value of
 // (row-tile pair ip, column tile jt) rounds to zero. Every role goes through the mask for itself, a
-// word of 32 tiles at a time; the issuers take the stages as they come and need the number of
-// tiles alone. Tile by tile, in one kernel for both cases: 0.260 ms a launch for 16 far-apart clusters
-// (N = 65,536, d = 8, 17 columns, 1 tile in 16 evaluated) and, for 64 clusters, d = 3, 336 us a call at
-// N = 65,536 and 992 at 131,072; like this 0.116 ms, 170 and 318 us.
+// word of 32 tiles at a time; the issuers and the epilogues take the stages as they come and need
+// the number of tiles alone (but for Matern-1/2's diagonal). Tile by tile, in one kernel for both
+// cases: 0.260 ms a launch for 16 far-apart clusters (N = 65,536, d = 8, 17 columns, 1 tile in 16
+// evaluated) and, for 64 clusters, d = 3, 336 us a call at N = 65,536 and 992 at 131,072; like this
+// 0.116 ms, 170 and 318 us.
 
 // Evaluated column tiles of pair ip in [j0, j1).
 template <int SKIP>
@@ -217,8 +217,7 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x, ++ic) {
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
-        const int xb = p.xi_bufs == 2 ? (ic & 1) : 0;
-        const int use = p.xi_bufs == 2 ? (ic >> 1) : ic;   // earlier uses of this buffer
+        const int xb = ic & 1, use = ic >> 1;   // earlier uses of this buffer
         if (use >= 1 && !ptx::mbar_wait(&bars.xi_empty[xb], (use - 1) & 1, p.limit_ns)) { ok = false; break; }
         uint8_t* sX = sXi + (uint32_t)xb * 2u * xbytes;
         ptx::mbar_arrive_expect_tx(&bars.xi_full[xb], 2u * xbytes);
@@ -248,10 +247,9 @@ __device__ void tp_producer(const TpParams& p, const CUtensorMap* tmA, const CUt
         const uint32_t first = fills > S ? fills - S : 0;
 #pragma unroll 1
         for (uint32_t f = first; f < fills; ++f) ptx::mbar_wait(&bars.full[f % S], (f / S) & 1, p.limit_ns);
-        const uint32_t nb = (uint32_t)p.xi_bufs;
 #pragma unroll 1
-        for (uint32_t q = xi_loads > nb ? xi_loads - nb : 0; q < xi_loads; ++q)
-            ptx::mbar_wait(&bars.xi_full[q % nb], (q / nb) & 1, p.limit_ns);
+        for (uint32_t q = xi_loads > 2 ? xi_loads - 2 : 0; q < xi_loads; ++q)
+            ptx::mbar_wait(&bars.xi_full[q & 1], (q >> 1) & 1, p.limit_ns);
     }
 }
 
@@ -311,8 +309,8 @@ struct TpSIssue {
             int ip, sp, j0, j1;
             item_range(p, item, ip, sp, j0, j1);
             left = tile_count<SKIP>(p, ip, j0, j1);
-            xb = p.xi_bufs == 2 ? (int)(ic & 1u) : 0;
-            ok = ok && warp_wait(&bars.xi_full[xb], (p.xi_bufs == 2 ? ic >> 1 : ic) & 1u, p.limit_ns);
+            xb = (int)(ic & 1u);
+            ok = ok && warp_wait(&bars.xi_full[xb], (ic >> 1) & 1u, p.limit_ns);
             ++ic;
         }
     }
@@ -520,9 +518,10 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
         int ip, sp, j0, j1;
         item_range(p, item, ip, sp, j0, j1);
         const int it = 2 * ip + tl;   // this warpgroup's row tile
-        const bool any = !SKIP || next_tile<SKIP>(p, ip, j0, j1) < j1;
+        const int tiles = tile_count<SKIP>(p, ip, j0, j1);
 #pragma unroll 1
-        for (int jt = next_tile<SKIP>(p, ip, j0, j1); jt < j1; jt = next_tile<SKIP>(p, ip, jt + 1, j1)) {
+        for (int n = tiles, jt = j0 - 1; n > 0; --n) {
+            if constexpr (KIND == GP_KERNEL_MATERN12) jt = next_tile<SKIP>(p, ip, jt + 1, j1);   // (the diagonal)
             const bool dtile = (KIND == GP_KERNEL_MATERN12) && p.diag && (jt == it);
 #pragma unroll
             for (int h = 0; h < H; ++h) {
@@ -594,7 +593,7 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
             }
         }
         // O read-out: lanes are rows of the tile; this warpgroup's half of the right-hand sides.
-        if (any) {
+        if (tiles > 0) {
             ok = ok && warp_wait(&bars.o_full[tl], oph, p.limit_ns);
             oph ^= 1u;
         }
@@ -606,7 +605,7 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
 #pragma unroll 1
         for (int c = c0; c < c1; c += 8) {   // warp-uniform
             uint32_t oh[8], ol[8];
-            if (any) {
+            if (tiles > 0) {
                 ptx::tmem_ld8(tO + (uint32_t)c, oh);
                 ptx::tmem_ld8(tO + (uint32_t)(p.lo_off + c), ol);
                 ptx::tmem_wait_ld();
@@ -847,7 +846,8 @@ cudaError_t launch_tp_typed(const TcPlan& plan, const TpParams& prm, const CUten
 }  // namespace
 
 // The operand sets this engine takes (rp: right-hand sides padded to 16, hi and
-// lo padded separately); the others run on the one-tile engine.
+// lo padded separately); the others run on the one-tile engine.  At k_pad = 64 the line at 64
+// columns dates from when P took shared memory; three stages of 48 KB would fit beyond it now.
 bool tp_supported(int k_pad, int R_pad, int vsplit) {
     const int rp = R_pad * (1 + vsplit);
     return k_pad <= 64 && rp <= (k_pad == 64 ? 64 : 128) && rp % 32 == 0;
@@ -868,8 +868,8 @@ TcPlan tp_plan(const Ctx* ctx, int64_t Nr, int64_t Nc, int R, int k_pad, int vsp
     p.Nc_pad = (int64_t)p.n_jt * kBN;
     const int G = ctx->num_sms > 0 ? ctx->num_sms : 1;
     // Column split minimising the busiest CTA's work (waves x tiles per item
-    // plus about two tiles of per-item cost) plus the reduction, which always
-    // runs here (it also sums the hi and lo rows).
+    // plus about two tiles of per-item cost) plus the reduction of the splits' hi and
+    // lo rows (counted for one split too, which writes its output itself).
     int best = 1;
     double best_cost = 1e300;
     const int max_split = p.n_jt < 16 ? p.n_jt : 16;
@@ -906,7 +906,6 @@ int launch_kmvm_tp(Ctx* ctx, const TcPlan& plan, const OperandLayout& L, const M
     const TpSmem m = tp_smem(plan.k_pad, plan.rv);
     if (m.stages < 2) return GP_ERR_UNSUPPORTED;
     prm.stages = m.stages;
-    prm.xi_bufs = m.xi_bufs;
     prm.sm = m;
     prm.diag = a.diag_coef != 0.0f ? 1 : 0;
     prm.ld_part = plan.Nr_pad;

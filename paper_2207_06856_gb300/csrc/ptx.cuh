@@ -25,9 +25,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void fence_mbar_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-__device__ __forceinline__ void fence_proxy_async_smem() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -161,19 +158,9 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uin
         "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// The same, issued by one elected lane of a converged warp (elect.sync): the
+// A from TMEM (.ts), issued by one elected lane of a converged warp (elect.sync): the
 // whole warp runs the issue loop, so addresses and descriptors stay
 // warp-uniform, and exactly one lane issues the instruction.
-__device__ __forceinline__ void mma_f16_ss_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                 uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 __device__ __forceinline__ void mma_f16_ts_elect(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                                  uint32_t accumulate) {
     asm volatile(
@@ -281,19 +268,8 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 
 // Shared-memory matrix descriptor (tcgen05): start address, leading / stride
 // byte offsets (16-byte units), fixed version bits 46-48 = 0b001, swizzle
-// mode in bits 61-63 (0 none, 2 = 128B, 4 = 64B, 6 = 32B).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes,
-                                              uint32_t swizzle_code) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)(swizzle_code & 7u) << 61;
-    return d;
-}
-// The same descriptor split into a constant high word and a low word that
-// only depends on the start address: lo = (addr >> 4) | (lbo >> 4) << 16.
+// mode in bits 61-63 (0 none, 2 = 128B, 4 = 64B, 6 = 32B); split into a constant high word and a
+// low word that only depends on the start address: lo = (addr >> 4) | (lbo >> 4) << 16.
 __device__ __forceinline__ uint32_t smem_desc_hi(uint32_t sbo_bytes, uint32_t swizzle_code) {
     return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | ((swizzle_code & 7u) << 29);
 }
