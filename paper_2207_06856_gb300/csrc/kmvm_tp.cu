@@ -44,8 +44,8 @@
 // With the FP32 value product (no P, no O) each row tile has two 128-column buffers.
 //
 // N = 65,536, d = 8, 17 columns, RBF, ms per launch (P in shared memory, one S and
-// one value-product issuer -> this form): FP16 tile 0.774 -> 0.621, hi + lo tile and
-// inputs 1.45 -> 0.88, of which 0.43 is the special-function time of one ex2 a pair.
+// one value-product issuer -> this form): FP16 tile 0.774 -> 0.611, hi + lo tile and
+// inputs 1.45 -> 0.867, of which 0.43 is the special-function time of one ex2 a pair.
 // With HS (GP_MVM_HALF_EXP) the S product accumulates in FP16 and the
 // epilogue evaluates 2^s in FP16 pairs.
 //
@@ -432,7 +432,7 @@ __device__ void tp_issuer_s(const TpParams& p, TpBarriers& bars, const uint8_t* 
 // row tile's epilogue warps have read it (p_empty, one arrival per warp). Here the waits are
 // mbarriers with the suspend-time hint on both sides: this epilogue is bound by issue slots and
 // registers, and one named barrier more in its loop spilled. N = 65,536, d = 8, hi + lo inputs, RBF, us
-// a call for 1, 2 and 4 columns: named barrier 795 / 1,203 / 2,171, this form 770 / 1,138 / 2,089.
+// a call for 1, 2 and 4 columns: named barrier 795 / 1,203 / 2,171, this form 769 / 1,137 / 2,077.
 template <int NG, int SKIP>
 __device__ void tp_issuer_spv(const TpParams& p, TpBarriers& bars, const uint8_t* sSt, const uint8_t* sXi,
                               uint32_t xbytes, uint32_t stage_bytes, uint32_t tmem, uint32_t id_s, uint32_t w) {
@@ -643,8 +643,8 @@ __device__ void tp_epilogue(const TpParams& p, TpBarriers& bars, uint32_t tmem, 
 // with FP32 FMAs, v_j read in FP32 from the stage (TMA box of 128 columns x 4
 // rows; this warpgroup's 64 columns; broadcast 16-byte reads).  No P and no
 // value-product MMAs: no rounding of the kernel values, and
-// one column takes 770 us a call against 867 on the hi + lo tile (N = 65,536, d = 8, RBF;
-// two 1,137 and four 2,088, where the hi + lo tile's time hardly changes).  Each warp releases
+// one column takes 769 us a call against 850 on the hi + lo tile (N = 65,536, d = 8, RBF;
+// two 1,137 and four 2,077, where the hi + lo tile's time hardly changes).  Each warp releases
 // the stage after its reads (16 arrivals), and writes its row sums of the item
 // to the partial rows ch * R + r, which the split reduction adds up.
 template <int KIND, int RN, int SKIP>
